@@ -348,7 +348,8 @@ int fewha_batch_launch(void *batch, cudaStream_t stream);
  *   3x3 cross-correlation with zero padding; act = ReLU if relu != 0; w is
  *   Cout x Cin x 3 x 3 (row-major), bias may be NULL.
  * fewha_conv3x3_bwd_data: gin = adjoint of that convolution (no bias, no act)
- *   applied to gout.
+ *   applied to gout.  fewha_conv3x3_bwd_data_relu: the same, then 0 where
+ *   act <= 0 (act laid out like gin, the ReLU output; NULL: no mask).
  * fewha_conv3x3_bwd_weight: gw (Cout x Cin x 9) and gb (Cout) of
  *   sum_b,co,y,x gout * out; written, or added when accumulate != 0;
  *   workspace: fewha_conv3x3_wgrad_workspace(...) floats; deterministic.
@@ -390,6 +391,9 @@ int fewha_conv3x3_fwd(const float *in, long in_bs, long in_cs, int Cin, const fl
 int fewha_conv3x3_fwd_tc(const float *in, long in_bs, long in_cs, int Cin, const float *w, const float *bias,
                          float *out, long out_bs, long out_cs, int Cout, int B, int H, int W, int relu,
                          int *status_dev, cudaStream_t s);
+int fewha_conv3x3_bwd_data_relu(const float *gout, long gout_bs, long gout_cs, int Cout, const float *w,
+                                const float *act, float *gin, long gin_bs, long gin_cs, int Cin, int B, int H, int W,
+                                cudaStream_t s);
 int fewha_conv3x3_bwd_data(const float *gout, long gout_bs, long gout_cs, int Cout, const float *w, float *gin,
                            long gin_bs, long gin_cs, int Cin, int B, int H, int W, cudaStream_t s);
 long fewha_conv3x3_wgrad_workspace(int Cin, int Cout, int B, int H, int W);

@@ -159,6 +159,7 @@ def load_library(path=LIB_PATH):
     learned = {
         "fewha_conv3x3_fwd": [vp, L, L, I, vp, vp, vp, L, L, I, I, I, I, I, vp],
         "fewha_conv3x3_fwd_tc": [vp, L, L, I, vp, vp, vp, L, L, I, I, I, I, I, vp, vp],
+        "fewha_conv3x3_bwd_data_relu": [vp, L, L, I, vp, vp, vp, L, L, I, I, I, I, vp],
         "fewha_conv3x3_bwd_data": [vp, L, L, I, vp, vp, L, L, I, I, I, I, vp],
         "fewha_conv3x3_bwd_weight": [vp, L, L, I, vp, L, L, I, I, I, I, vp, vp, I, vp, vp],
         "fewha_relu_bwd": [vp, vp, L, vp],
@@ -190,7 +191,7 @@ def exported_symbols():
             "fewha_batch_ctas", "fewha_batch_solve", "fewha_batch_destroy", "fewha_strerror",
             "fewha_batch_bind", "fewha_batch_launch", "fewha_batch_create_rounds", "fewha_n_actuators", "fewha_fit",
             "fewha_pol_slopes", "fewha_control",
-            "fewha_apply_op_multi", "fewha_conv3x3_fwd", "fewha_conv3x3_bwd_data",
+            "fewha_apply_op_multi", "fewha_conv3x3_fwd", "fewha_conv3x3_bwd_data", "fewha_conv3x3_bwd_data_relu",
             "fewha_conv3x3_wgrad_workspace", "fewha_conv3x3_bwd_weight", "fewha_relu_bwd",
             "fewha_mse_grad", "fewha_adam_step", "fewha_scale", "fewha_learned_targets",
             "fewha_deflate_warm_start", "fewha_mcao_create", "fewha_mcao_n_actuators", "fewha_mcao_fit",

@@ -163,19 +163,17 @@ class ConvNet:
             self._ck(lib.fewha_conv3x3_bwd_weight(C.c_void_p(h2.data_ptr()), 32 * hw, hw, c2, gyp, hw, gy.stride(0),
                                                   c3, cnt, nl, nl, self._p(self.grad, "w3"),
                                                   self._p(self.grad, "b3"), acc, work, s), "wgrad3")
-            self._ck(lib.fewha_conv3x3_bwd_data(gyp, hw, gy.stride(0), c3, self._p(self.param, "w3"),
-                                                C.c_void_p(ga.data_ptr()), 32 * hw, hw, c2, cnt, nl, nl, s), "dgrad3")
-            self._ck(lib.fewha_relu_bwd(C.c_void_p(h2.data_ptr()), C.c_void_p(ga.data_ptr()), ga.numel(), s),
-                     "relu2")
+            self._ck(lib.fewha_conv3x3_bwd_data_relu(gyp, hw, gy.stride(0), c3, self._p(self.param, "w3"),
+                                                     C.c_void_p(h2.data_ptr()), C.c_void_p(ga.data_ptr()), 32 * hw,
+                                                     hw, c2, cnt, nl, nl, s), "dgrad3")
             self._ck(lib.fewha_conv3x3_bwd_weight(C.c_void_p(h1.data_ptr()), 32 * hw, hw, c1,
                                                   C.c_void_p(ga.data_ptr()), 32 * hw, hw, c2, cnt, nl, nl,
                                                   self._p(self.grad, "w2"), self._p(self.grad, "b2"), acc, work, s),
                      "wgrad2")
-            self._ck(lib.fewha_conv3x3_bwd_data(C.c_void_p(ga.data_ptr()), 32 * hw, hw, c2,
-                                                self._p(self.param, "w2"), C.c_void_p(gb.data_ptr()), 32 * hw, hw,
-                                                c1, cnt, nl, nl, s), "dgrad2")
-            self._ck(lib.fewha_relu_bwd(C.c_void_p(h1.data_ptr()), C.c_void_p(gb.data_ptr()), gb.numel(), s),
-                     "relu1")
+            self._ck(lib.fewha_conv3x3_bwd_data_relu(C.c_void_p(ga.data_ptr()), 32 * hw, hw, c2,
+                                                     self._p(self.param, "w2"), C.c_void_p(h1.data_ptr()),
+                                                     C.c_void_p(gb.data_ptr()), 32 * hw, hw, c1, cnt, nl, nl, s),
+                     "dgrad2")
             self._ck(lib.fewha_conv3x3_bwd_weight(C.c_void_p(x_ptr + 4 * off), hw, x_cs, c0,
                                                   C.c_void_p(gb.data_ptr()), 32 * hw, hw, c1, cnt, nl, nl,
                                                   self._p(self.grad, "w1"), self._p(self.grad, "b1"), acc, work, s),

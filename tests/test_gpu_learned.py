@@ -81,6 +81,32 @@ def test_conv_forward_and_gradients(lib, B, Cin, Cout, H, W):
     assert rel(gw.cpu().numpy(), 2 * rw) < 1e-5 and rel(gb.cpu().numpy(), 2 * rb) < 1e-5
 
 
+@pytest.mark.parametrize("B,Cin,Cout,H,W", [(1, 1, 1, 1, 1), (1, 32, 32, 17, 15), (5, 33, 9, 16, 33), (2, 5, 8, 7, 50),
+                                            (90, 4, 40, 40, 24)])
+def test_conv_gradients_at_tile_and_channel_edges(lib, B, Cin, Cout, H, W):
+    """Channel blocks with a remainder, images within and just past a tile, more tiles than CTAs; the data
+    gradient with the ReLU's mask against its two steps.  The weight gradient sums B H W products in FP32 per
+    tile and FP64 across CTAs, and its terms cancel: the bound is 1e-5 of the root of the sums of squares."""
+    _, L = lib
+    rng = np.random.default_rng(B + Cin)
+    x, w, g = rng.standard_normal((B, Cin, H, W)), rng.standard_normal((Cout, Cin, 3, 3)), rng.standard_normal(
+        (B, Cout, H, W))
+    xd, wd, gd = dev(x), dev(w), dev(g)
+    hw = H * W
+    act = torch.relu(xd)
+    gin = torch.full((B, Cin, H, W), 7.0, device="cuda")
+    assert L.fewha_conv3x3_bwd_data_relu(ptr(gd), Cout * hw, hw, Cout, ptr(wd), ptr(act), ptr(gin), Cin * hw, hw, Cin,
+                                         B, H, W, S()) == 0
+    assert rel(gin.cpu().numpy(), OL.conv3x3_bwd_data(g, w) * (act.cpu().numpy() > 0)) < 1e-5
+    ws = torch.empty(L.fewha_conv3x3_wgrad_workspace(Cin, Cout, B, H, W), device="cuda")
+    gw, gb = torch.full((Cout, Cin, 3, 3), 7.0, device="cuda"), torch.full((Cout,), 7.0, device="cuda")
+    assert L.fewha_conv3x3_bwd_weight(ptr(xd), Cin * hw, hw, Cin, ptr(gd), Cout * hw, hw, Cout, B, H, W,
+                                      ptr(gw), ptr(gb), 0, ptr(ws), S()) == 0
+    rw, rb = OL.conv3x3_bwd_weight(x, g)
+    scale = np.sqrt(B * hw)
+    assert np.abs(gw.cpu().numpy() - rw).max() < 1e-5 * scale and np.abs(gb.cpu().numpy() - rb).max() < 1e-5 * scale
+
+
 def test_conv_strided_channels(lib):
     """Channels as whole vectors (stride n, and -n over a ring, newest first)."""
     _, L = lib
