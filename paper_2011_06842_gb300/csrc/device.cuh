@@ -79,6 +79,7 @@ struct Geo {
     int lay_n[FEWHA_MAX_LAYERS], lay_J[FEWHA_MAX_LAYERS];
     long lay_off[FEWHA_MAX_LAYERS + 1];
     long ll_off[FEWHA_MAX_LAYERS + 1];  // (n_l/2)^2 blocks: level-1 approximation scratch
+    int depth;                  // split form: finest wavelet levels tiled over all CTAs (split_depth)
     T inv_delta[FEWHA_MAX_LAYERS];
     int n_taps;
     T h[kMaxT], g[kMaxT];
@@ -128,7 +129,7 @@ struct __align__(16) Args {
     S *psi;          // [G][m*m] Gamma^T C Gamma P_g (...) per guide star
     T *u;            // [n]  P^T psi (layer nodal adjoint)
     T *wq;           // [n]  W^{-T} u / delta (operator output before + alpha D p)
-    T *ll;           // [sum (n_l/2)^2] level-1 approximation of each layer (split transforms)
+    T *ll;           // [sum (n_l/2)^2] level-1 approximation of each layer, then [sum (n_l/4)^2] level-2 (split transforms)
     // working-precision (T) buffers of the residual replacement's operator
     // application: the nodal layers and adjoint wavefronts are stored in T
     // there even when S is narrower (== nodal / psi when S is T)

@@ -240,12 +240,12 @@ __global__ void __launch_bounds__(kThreads, 1) k_rhs_gather(const __grid_constan
 }
 
 // R3: the finest analysis level of u (split form), then b, r0 and P^T r0
-template <typename T, typename S>
+template <typename T, typename S, int LV>
 __global__ void __launch_bounds__(kThreads, 1) k_rhs_D1(const __grid_constant__ Args<T, S> Ap)
 {
     FEWHA_PHASE_GUARD
     (void)sc;
-    if (!A.rhs_in_state) phase_D1<T, S>(A, dyn_smem<T>());
+    if (!A.rhs_in_state) phase_D1<LV>(A, dyn_smem<T>());
 }
 
 template <typename T, typename S>
@@ -273,12 +273,12 @@ __global__ void __launch_bounds__(kThreads, 1) k_UA1(const __grid_constant__ Arg
     phase_UA1<T, S>(A, b, k, dyn_smem<T>(), sc, sred);
 }
 
-template <typename T, typename S>
+template <typename T, typename S, int LV>
 __global__ void __launch_bounds__(kThreads, 1) k_A2(const __grid_constant__ Args<T, S> Ap, int k)
 {
     FEWHA_PHASE_GUARD
     (void)sc;
-    phase_A2<T, S>(A, b, k, dyn_smem<T>());
+    phase_A2<LV>(A, b, k, dyn_smem<T>());
 }
 
 template <typename T, typename S>
@@ -298,12 +298,12 @@ __global__ void __launch_bounds__(kThreads, 1) k_C(const __grid_constant__ Args<
     phase_C<T, S>(A, b, k, dyn_smem<T>(), sc);
 }
 
-template <typename T, typename S>
+template <typename T, typename S, int LV>
 __global__ void __launch_bounds__(kThreads, 1) k_D1(const __grid_constant__ Args<T, S> Ap, int k)
 {
     FEWHA_PHASE_GUARD
     (void)sc;
-    phase_D1<T, S>(A, dyn_smem<T>());
+    phase_D1<LV>(A, dyn_smem<T>());
 }
 
 template <typename T, typename S>
@@ -323,13 +323,13 @@ __global__ void __launch_bounds__(kThreads, 1) k_TU(const __grid_constant__ Args
     phase_TU<T>(*TrView<T, S>::get(A), dyn_smem<T>());
 }
 
-template <typename T, typename S>
+template <typename T, typename S, int LV>
 __global__ void __launch_bounds__(kThreads, 1) k_TA2(const __grid_constant__ Args<T, S> Ap)
 {
     FEWHA_PHASE_GUARD
     (void)sc;
     const Args<T, T> &V = *TrView<T, S>::get(A);
-    phase_fine_synth<T, T>(V, V.c, dyn_smem<T>());
+    phase_fine_synth<LV>(V, V.c, dyn_smem<T>());
 }
 
 template <typename T, typename S>
@@ -348,12 +348,12 @@ __global__ void __launch_bounds__(kThreads, 1) k_TC(const __grid_constant__ Args
     band_gather<T, T>(*TrView<T, S>::get(A), dyn_smem<T>());
 }
 
-template <typename T, typename S>
+template <typename T, typename S, int LV>
 __global__ void __launch_bounds__(kThreads, 1) k_TD1(const __grid_constant__ Args<T, S> Ap)
 {
     FEWHA_PHASE_GUARD
     (void)sc;
-    phase_D1<T, T>(*TrView<T, S>::get(A), dyn_smem<T>());
+    phase_D1<LV>(*TrView<T, S>::get(A), dyn_smem<T>());
 }
 
 template <typename T, typename S>
@@ -385,7 +385,7 @@ __device__ __forceinline__ bool true_residual_phases(const Args<T, T> &V, const 
                                                      int rank, int &ti)
 {
     T *sm = dyn_smem<T>();
-    const bool split = split_levels(V);
+    const bool split = split_levels(V), deep = split && split_depth(V.geo) > 1;
     auto sync = [&](int tag) -> bool {
         unsigned long long *slot = (V.trace && ti < V.trace_cap) ? V.trace + 4 * ti : nullptr;
         if (slot && rank == 0 && threadIdx.x == 0) slot[3] = (unsigned long long)tag;
@@ -394,8 +394,12 @@ __device__ __forceinline__ bool true_residual_phases(const Args<T, T> &V, const 
     };
     phase_TU<T>(V, sm);
     if (!sync(20)) return false;
+    if (deep) {
+        phase_fine_synth<1>(V, V.c, sm);
+        if (!sync(26)) return false;
+    }
     if (split) {
-        phase_fine_synth<T, T>(V, V.c, sm);
+        phase_fine_synth(V, V.c, sm);
         if (!sync(21)) return false;
     }
     wfs_phase<T, T, false>(V, sm);
@@ -403,8 +407,12 @@ __device__ __forceinline__ bool true_residual_phases(const Args<T, T> &V, const 
     band_gather<T, T>(V, sm);
     if (!sync(23)) return false;
     if (split) {
-        phase_D1<T, T>(V, sm);
+        phase_D1(V, sm);
         if (!sync(24)) return false;
+    }
+    if (deep) {
+        phase_D1<1>(V, sm);
+        if (!sync(27)) return false;
     }
     phase_TE<T>(V, b, k, sm, sred);
     return sync(25);
@@ -433,6 +441,7 @@ __device__ void solve_body(const Args<T, S> &A, Scal &sc, double *sred)
     };
     int K = A.max_iter;
     const bool split = split_levels(A);  // uniform over the instance's CTAs
+    const bool deep = split && split_depth(A.geo) > 1;
     const Args<T, T> *V = nullptr;  // residual replacement's view of the arguments
     if constexpr (TR) V = TrView<T, S>::get(A);
     trace_begin(A.trace != nullptr);
@@ -445,8 +454,12 @@ __device__ void solve_body(const Args<T, S> &A, Scal &sc, double *sred)
         if (b.kv > 0 && rank == A.ncta - 1) phase_factor<T, S>(A, b, sc);
         if ((rhs || b.kv > 0) && !sync(2)) break;
         if (split && rhs) {
-            phase_D1<T, S>(A, sm);  // the finest analysis level of u
+            phase_D1(A, sm);  // the finest analysis level of u
             if (!sync(6)) break;
+            if (deep) {
+                phase_D1<1>(A, sm);
+                if (!sync(7)) break;
+            }
         }
         phase_rhs_update<T, S, RIS>(A, b, sm, sred);  // b, r0 and P^T r0
         if (!sync(3)) break;
@@ -462,8 +475,12 @@ __device__ void solve_body(const Args<T, S> &A, Scal &sc, double *sred)
                 break;
             }
             if (!sync(10)) break;
+            if (deep) {
+                phase_A2<1>(A, b, k, sm);
+                if (!sync(17)) break;
+            }
             if (split) {
-                phase_A2<T, S>(A, b, k, sm);
+                phase_A2(A, b, k, sm);
                 if (!sync(16)) break;
             }
             {
@@ -478,8 +495,12 @@ __device__ void solve_body(const Args<T, S> &A, Scal &sc, double *sred)
             }
             if (!sync(13)) break;
             if (split) {
-                phase_D1<T, S>(A, sm);
+                phase_D1(A, sm);
                 if (!sync(14)) break;
+            }
+            if (deep) {
+                phase_D1<1>(A, sm);
+                if (!sync(18)) break;
             }
             phase_D2E<T, S>(A, b, k, sm, sred, &sc.alpha);
             if (!sync(15)) break;
@@ -892,6 +913,17 @@ struct Impl : ImplBase {
             const long h = P.geom.layers[l].n / 2;
             G.ll_off[l + 1] = G.ll_off[l] + h * h;
         }
+        // two tiled levels where a layer CTA's block would be 64^2 in FP64 (split_depth)
+        {
+            int nmax = 0;
+            bool ok = sizeof(T) == 8;
+            for (int l = 0; l < P.L; l++) {
+                const fewha_layer &ly = P.geom.layers[l];
+                nmax = std::max(nmax, ly.n);
+                ok = ok && ly.J >= 2 && ly.n >= 32;
+            }
+            G.depth = ok && nmax >= 128 ? 2 : 1;
+        }
         G.n_taps = (int)P.taps.size();
         for (int t = 0; t < kMaxT; t++) {
             G.h[t] = t < G.n_taps ? (T)P.taps[t] : T(0);
@@ -944,7 +976,7 @@ struct Impl : ImplBase {
         }
         if ((st = alloc((size_t)P.n, &base.nodal)) || (st = alloc((size_t)P.n, &base.u)) ||
             (st = alloc((size_t)P.n, &base.wq)) ||
-            (st = alloc((size_t)P.psi_off[P.G], &base.psi)) || (st = alloc((size_t)P.n / 4 + 1, &base.ll)) ||
+            (st = alloc((size_t)P.psi_off[P.G], &base.psi)) || (st = alloc((size_t)P.n / 4 + P.n / 16 + 1, &base.ll)) ||
             (st = alloc((size_t)kSlots * kMaxCtas, &base.part)) || (st = alloc((size_t)1, &base.rec)))
             return st;
         if constexpr (std::is_same<T, S>::value) {
@@ -991,22 +1023,27 @@ struct Impl : ImplBase {
         CK(setattr((const void *)k_fdwt<T, S, false>));
         CK(setattr((const void *)k_fdwt<T, S, true>));
         CK(setattr((const void *)k_rhs_wfs<T, S>));
-        CK(setattr((const void *)k_rhs_D1<T, S>));
+        CK(setattr((const void *)k_rhs_D1<T, S, 0>));
+        CK(setattr((const void *)k_rhs_D1<T, S, 1>));
         CK(setattr((const void *)k_rhs_update<T, S>));
         CK(setattr((const void *)k_rhs_gather<T, S>));
         CK(setattr((const void *)k_init<T, S>));
         CK(setattr((const void *)k_UA1<T, S>));
-        CK(setattr((const void *)k_A2<T, S>));
+        CK(setattr((const void *)k_A2<T, S, 0>));
+        CK(setattr((const void *)k_A2<T, S, 1>));
         CK(setattr((const void *)k_B<T, S>));
         CK(setattr((const void *)k_C<T, S>));
-        CK(setattr((const void *)k_D1<T, S>));
+        CK(setattr((const void *)k_D1<T, S, 0>));
+        CK(setattr((const void *)k_D1<T, S, 1>));
         CK(setattr((const void *)k_D2E<T, S>));
         CK(setattr((const void *)k_finish<T, S>));
         CK(setattr((const void *)k_TU<T, S>));
-        CK(setattr((const void *)k_TA2<T, S>));
+        CK(setattr((const void *)k_TA2<T, S, 0>));
+        CK(setattr((const void *)k_TA2<T, S, 1>));
         CK(setattr((const void *)k_TB<T, S>));
         CK(setattr((const void *)k_TC<T, S>));
-        CK(setattr((const void *)k_TD1<T, S>));
+        CK(setattr((const void *)k_TD1<T, S, 0>));
+        CK(setattr((const void *)k_TD1<T, S, 1>));
         CK(setattr((const void *)k_TE<T, S>));
         CK(setattr((const void *)k_solve_persistent<T, S, false>));
         CK(setattr((const void *)k_solve_persistent<T, S, true>));
@@ -1515,24 +1552,30 @@ struct Impl : ImplBase {
                 CK(cudaLaunchKernelEx(&cfg, k_solve_persistent<T, S, false>, A));
             return launch_check();
         }
+        const bool deep = A.geo.depth > 1 && ncta >= 2 * P.L;  // split_levels, split_depth
         k_rhs_wfs<T, S><<<ncta, kThreads, smem, s>>>(A);
         k_rhs_gather<T, S><<<ncta, kThreads, smem, s>>>(A);
-        k_rhs_D1<T, S><<<ncta, kThreads, smem, s>>>(A);
+        k_rhs_D1<T, S, 0><<<ncta, kThreads, smem, s>>>(A);
+        if (deep) k_rhs_D1<T, S, 1><<<ncta, kThreads, smem, s>>>(A);
         k_rhs_update<T, S><<<ncta, kThreads, smem, s>>>(A);
         k_init<T, S><<<ncta, kThreads, smem, s>>>(A);
         for (int k = 0; k < A.max_iter; k++) {
             k_UA1<T, S><<<ncta, kThreads, smem, s>>>(A, k);
-            k_A2<T, S><<<ncta, kThreads, smem, s>>>(A, k);
+            if (deep) k_A2<T, S, 1><<<ncta, kThreads, smem, s>>>(A, k);
+            k_A2<T, S, 0><<<ncta, kThreads, smem, s>>>(A, k);
             k_B<T, S><<<ncta, kThreads, smem, s>>>(A, k);
             k_C<T, S><<<ncta, kThreads, smem, s>>>(A, k);
-            k_D1<T, S><<<ncta, kThreads, smem, s>>>(A, k);
+            k_D1<T, S, 0><<<ncta, kThreads, smem, s>>>(A, k);
+            if (deep) k_D1<T, S, 1><<<ncta, kThreads, smem, s>>>(A, k);
             k_D2E<T, S><<<ncta, kThreads, smem, s>>>(A, k);
             if (A.true_res_every > 0 && (k + 1) % A.true_res_every == 0) {
                 k_TU<T, S><<<ncta, kThreads, smem, s>>>(A);
-                k_TA2<T, S><<<ncta, kThreads, smem, s>>>(A);
+                if (deep) k_TA2<T, S, 1><<<ncta, kThreads, smem, s>>>(A);
+                k_TA2<T, S, 0><<<ncta, kThreads, smem, s>>>(A);
                 k_TB<T, S><<<ncta, kThreads, smem, s>>>(A);
                 k_TC<T, S><<<ncta, kThreads, smem, s>>>(A);
-                k_TD1<T, S><<<ncta, kThreads, smem, s>>>(A);
+                k_TD1<T, S, 0><<<ncta, kThreads, smem, s>>>(A);
+                if (deep) k_TD1<T, S, 1><<<ncta, kThreads, smem, s>>>(A);
                 k_TE<T, S><<<ncta, kThreads, smem, s>>>(A, k);
             }
         }

@@ -243,11 +243,33 @@ __device__ __forceinline__ void phase_init(const Args<T, S> &A, const Basis &b, 
 }
 
 // ---------------------------------------------------------------------------
-// Element loops of the fused phases.  Every layer's top-left (n/2)^2 block (the
-// approximation part of the finest wavelet level) belongs to the layer's CTA,
-// which transforms it in shared memory; every other coefficient to the CTA
-// whose element range holds it.
+// Element loops of the fused phases.  Every layer's top-left (n/2^d)^2 block
+// (the approximation part of the d = split_depth finest wavelet levels)
+// belongs to the layer's CTA, which transforms it in shared memory; every
+// other coefficient to the CTA whose element range holds it.
 // ---------------------------------------------------------------------------
+// Finest levels that the split form tiles over all CTAs: one, or two in FP64
+// with layers of at least 128^2 (Geo::depth, set on the host).  A layer CTA has
+// about two FP64 FMAs per clock: the 64^2 block of a 128^2 layer keeps it ~26 us
+// in UA1 and again in D2E (8 operations per element of the update, 12 per
+// element and level of the transform), the 32^2 block a quarter of that, for one
+// more tiled phase and barrier on each side.  In FP32 the block is latency
+// bound and a phase with its barrier costs more than the level saves.
+template <typename T>
+__device__ __forceinline__ int split_depth(const Geo<T> &G)
+{
+    if constexpr (sizeof(T) == 8) return G.depth;
+    return 1;
+}
+
+// Approximation scratch of layer l at level t (1 or 2): (n_l >> t)^2, row-major.
+template <typename T, typename S>
+__device__ __forceinline__ T *ll_block(const Args<T, S> &A, int l, int t)
+{
+    const Geo<T> &G = A.geo;
+    return t == 1 ? A.ll + G.ll_off[l] : A.ll + G.ll_off[G.L] + (G.ll_off[l] >> 2);
+}
+
 template <typename T, typename F>
 __device__ __forceinline__ void for_detail_vectors(const Geo<T> &G, long lo, long hi, F body)
 {
@@ -256,7 +278,7 @@ __device__ __forceinline__ void for_detail_vectors(const Geo<T> &G, long lo, lon
     for (long e = lo + (long)threadIdx.x * W; e < hi; e += (long)blockDim.x * W) {
         while (e >= G.lay_off[l + 1]) l++;
         const long loc = e - G.lay_off[l];
-        const int h = G.lay_n[l] >> 1;
+        const int h = G.lay_n[l] >> split_depth(G);
         if ((int)(loc >> G.lay_lg[l]) < h && (int)(loc & (G.lay_n[l] - 1)) < h) continue;
         body(e);
     }
@@ -277,12 +299,12 @@ __device__ __forceinline__ bool split_levels(const Args<T, S> &A)
     return A.ncta >= 2 * A.geo.L;
 }
 
-// body(global element, index in the (n/2)^2 block), one W-vector per call
+// body(global element, index in the layer CTA's block), one W-vector per call
 template <typename T, typename F>
 __device__ __forceinline__ void for_block_vectors(const Geo<T> &G, int l, F body)
 {
     constexpr int W = VW<T>::W;
-    const int n = G.lay_n[l], h = n >> 1, lgh = G.lay_lg[l] - 1, nv = h * h / W;
+    const int d = split_depth(G), n = G.lay_n[l], h = n >> d, lgh = G.lay_lg[l] - d, nv = h * h / W;
     for (int v = threadIdx.x; v < nv; v += blockDim.x) {
         const int be = v * W;
         body(G.lay_off[l] + (long)(be >> lgh) * n + (be & (h - 1)), be);
@@ -341,7 +363,8 @@ __device__ __forceinline__ bool phase_UA1(const Args<T, S> &A, const Basis &b, i
         // red: [0] rz, [1] zq, [2] rp, [3] rr (E_{k-1}); [4..4+kv) Q^T z, [4+kK..) P^T r
         if (split && !A.recycle_all) {
             if (A.vrank() < G.L) {
-                const int l = A.vrank(), h = G.lay_n[l] >> 1, lgh = G.lay_lg[l] - 1, be = threadIdx.x * W;
+                const int d = split_depth(G), l = A.vrank(), h = G.lay_n[l] >> d, lgh = G.lay_lg[l] - d;
+                const int be = threadIdx.x * W;
                 if (be < h * h) pe = G.lay_off[l] + (long)(be >> lgh) * G.lay_n[l] + (be & (h - 1));
             } else {
                 long lo, hi;
@@ -452,7 +475,7 @@ __device__ __forceinline__ bool phase_UA1(const Args<T, S> &A, const Basis &b, i
     if (split) {
         // one layer per layer CTA (ncta >= 2L); the others take the details
         if (A.vrank() < G.L) {
-            const int l = A.vrank(), h = G.lay_n[l] >> 1, lgh = G.lay_lg[l] - 1;
+            const int d = split_depth(G), l = A.vrank(), h = G.lay_n[l] >> d, lgh = G.lay_lg[l] - d;
             for_block_vectors(G, l, [&](long e, int be) {
                 T p[W];
                 update(e, p);
@@ -461,8 +484,8 @@ __device__ __forceinline__ bool phase_UA1(const Args<T, S> &A, const Basis &b, i
                 for (int i = 0; i < W; i++) buf[s0 + i] = p[i];
             });
             __syncthreads();
-            idwt2<T>(buf, G.pingpong ? buf + h * (h + 1) : buf, lgh, G.lay_J[l] - 1, G);
-            T *ll = A.ll + G.ll_off[l];
+            idwt2<T>(buf, G.pingpong ? buf + h * (h + 1) : buf, lgh, G.lay_J[l] - d, G);
+            T *ll = ll_block(A, l, d);
             for (int v = threadIdx.x; v < h * h / W; v += blockDim.x) {
                 const int be = v * W, s0 = spad(be, lgh);
                 T x[W];
@@ -574,17 +597,22 @@ __device__ __forceinline__ bool phase_C(const Args<T, S> &A, const Basis &b, int
 // as the single-CTA transform (rows then columns for analysis, columns then
 // rows for synthesis).
 // ---------------------------------------------------------------------------
-constexpr int kFineTile = 16;
+// Geo::depth 2 tiles the next level the same way, from and to the level-1
+// approximation in A.ll, in tiles of kFineTile2 pairs (a quarter of the work:
+// the smaller tile keeps as many CTAs busy).
+constexpr int kFineTile = 16, kFineTile2 = 8;
 
 // Work item w -> layer l and tile origin (in coefficient pairs); false past the end.
-template <typename T>
+// of level LV (0 = finest)
+template <int LV, typename T>
 __device__ __forceinline__ bool fine_tile(const Geo<T> &G, int w, int &l, int &p0y, int &p0x)
 {
+    constexpr int TL = LV == 0 ? kFineTile : kFineTile2;
     for (l = 0; l < G.L; l++) {
-        const int h = G.lay_n[l] >> 1, nt = (h + kFineTile - 1) / kFineTile;
+        const int h = G.lay_n[l] >> (LV + 1), nt = (h + TL - 1) / TL;
         if (w < nt * nt) {
-            p0y = (w / nt) * kFineTile;
-            p0x = (w % nt) * kFineTile;
+            p0y = (w / nt) * TL;
+            p0x = (w % nt) * TL;
             return true;
         }
         w -= nt * nt;
@@ -593,22 +621,24 @@ __device__ __forceinline__ bool fine_tile(const Geo<T> &G, int w, int &l, int &p
 }
 
 // D1: level-1 analysis of u; the three detail bands are final coefficients of
-// W^{-T} u / delta (into wq), the approximation block goes to A.ll.
-template <typename T, typename S, int L>
+// W^{-T} u / delta (into wq), the approximation block goes to A.ll.  LV = 1: the
+// same of the level-1 approximation.
+template <typename T, typename S, int L, int LV>
 __device__ void fine_analysis(const Args<T, S> &A, T *sm)
 {
     const Geo<T> &G = A.geo;
     const Taps<T, L> tp = load_taps<T, L>(G);
     int l, p0y, p0x;
-    for (int w = A.vrank(); fine_tile(G, w, l, p0y, p0x); w += A.ncta) {
-        const int n = G.lay_n[l], h = n >> 1;
-        const int ty = min(kFineTile, h - p0y), tx = min(kFineTile, h - p0x);
+    constexpr int TL = LV == 0 ? kFineTile : kFineTile2;
+    for (int w = A.vrank(); fine_tile<LV>(G, w, l, p0y, p0x); w += A.ncta) {
+        const int n = G.lay_n[l], N = n >> LV, h = N >> 1;
+        const int ty = min(TL, h - p0y), tx = min(TL, h - p0x);
         const int IR = 2 * ty + L - 2, IC = 2 * tx + L - 2, MC = 2 * tx;
         T *in = sm, *mid = sm + IR * IC;
-        const T *u = A.u + G.lay_off[l];
+        const T *u = LV == 0 ? A.u + G.lay_off[l] : ll_block(A, l, 1);
         for (int e = threadIdx.x; e < IR * IC; e += blockDim.x) {
             const int r = e / IC, c = e - r * IC;
-            in[e] = ldcg(u + (long)((2 * p0y + r) & (n - 1)) * n + ((2 * p0x + c) & (n - 1)));
+            in[e] = ldcg(u + (long)((2 * p0y + r) & (N - 1)) * N + ((2 * p0x + c) & (N - 1)));
         }
         __syncthreads();
         for (int e = threadIdx.x; e < IR * tx; e += blockDim.x) {  // rows
@@ -626,7 +656,7 @@ __device__ void fine_analysis(const Args<T, S> &A, T *sm)
         __syncthreads();
         const T sc = G.inv_delta[l];
         T *wq = A.wq + G.lay_off[l];
-        T *ll = A.ll + G.ll_off[l];
+        T *ll = ll_block(A, l, LV + 1);
         for (int e = threadIdx.x; e < ty * MC; e += blockDim.x) {  // columns
             const int k = e / MC, c = e - k * MC;
             const T *x = mid + 2 * k * MC + c;
@@ -651,21 +681,23 @@ __device__ void fine_analysis(const Args<T, S> &A, T *sm)
 }
 
 // A2: level-1 synthesis of p_k's layers from the approximation block in A.ll
-// (A1) and p_k's three detail bands; nodal = W^{-1} p_k.
-template <typename T, typename S, int L>
+// (A1) and p_k's three detail bands; nodal = W^{-1} p_k.  LV = 1: level 2, from
+// its approximation and detail bands to the level-1 approximation.
+template <typename T, typename S, int L, int LV>
 __device__ void fine_synthesis(const Args<T, S> &A, const T *pk, T *sm)
 {
     constexpr int Lh = L / 2;
     const Geo<T> &G = A.geo;
     const Taps<T, L> tp = load_taps<T, L>(G);
     int l, p0y, p0x;
-    for (int w = A.vrank(); fine_tile(G, w, l, p0y, p0x); w += A.ncta) {
-        const int n = G.lay_n[l], h = n >> 1;
-        const int ty = min(kFineTile, h - p0y), tx = min(kFineTile, h - p0x);
+    constexpr int TL = LV == 0 ? kFineTile : kFineTile2;
+    for (int w = A.vrank(); fine_tile<LV>(G, w, l, p0y, p0x); w += A.ncta) {
+        const int n = G.lay_n[l], N = n >> LV, h = N >> 1;
+        const int ty = min(TL, h - p0y), tx = min(TL, h - p0x);
         const int WR = ty + Lh - 1, WC = tx + Lh - 1, Q = WR * WC;
         T *win = sm;              // [4][WR][WC]: LL, LH, HL, HH windows
         T *mid = sm + 4 * Q;      // [2 ty][2 WC]: columns synthesised, low-x then high-x
-        const T *ll = A.ll + G.ll_off[l];
+        const T *ll = ll_block(A, l, LV + 1);
         const T *pl = pk + G.lay_off[l];
         for (int e = threadIdx.x; e < 4 * Q; e += blockDim.x) {
             const int qd = e / Q, r = (e - qd * Q) / WC, c = e - qd * Q - r * WC;
@@ -698,6 +730,7 @@ __device__ void fine_synthesis(const Args<T, S> &A, const T *pk, T *sm)
         __syncthreads();
         const T sc = G.inv_delta[l];
         S *nodal = A.nodal + G.lay_off[l];
+        T *ll1 = ll_block(A, l, 1);
         for (int e = threadIdx.x; e < 2 * ty * 2 * tx; e += blockDim.x) {  // rows
             const int yy = e / (2 * tx), xx = e - yy * (2 * tx), j = xx >> 1, ex = xx & 1;
             const T *row = mid + yy * 2 * WC;
@@ -707,42 +740,49 @@ __device__ void fine_synthesis(const Args<T, S> &A, const T *pk, T *sm)
                 const int c = j + Lh - 1 - u;
                 x += tp.h[ex + 2 * u] * row[c] + tp.g[ex + 2 * u] * row[WC + c];
             }
-            nodal[(long)(2 * p0y + yy) * n + 2 * p0x + xx] = Cv<S>::st(x * sc);
+            const long o = (long)(2 * p0y + yy) * N + 2 * p0x + xx;
+            if constexpr (LV == 0)
+                nodal[o] = Cv<S>::st(x * sc);
+            else
+                ll1[o] = x;
         }
         __syncthreads();
     }
 }
 
-// The finest synthesis level of vector x, tiled over all CTAs (split form).
-template <typename T, typename S>
+// A tiled synthesis level of vector x over all CTAs (split form): LV = 0 the
+// finest, LV = 1 the one before it (split_depth 2 only).
+template <int LV = 0, typename T, typename S>
 __device__ __forceinline__ void phase_fine_synth(const Args<T, S> &A, const T *x, T *sm)
 {
-    if (!split_levels(A)) return;
+    if (!split_levels(A) || split_depth(A.geo) <= LV) return;
     switch (A.geo.n_taps) {
-    case 2: fine_synthesis<T, S, 2>(A, x, sm); break;
-    case 4: fine_synthesis<T, S, 4>(A, x, sm); break;
-    case 6: fine_synthesis<T, S, 6>(A, x, sm); break;
-    default: fine_synthesis<T, S, 8>(A, x, sm); break;
+    case 2: fine_synthesis<T, S, 2, LV>(A, x, sm); break;
+    case 4: fine_synthesis<T, S, 4, LV>(A, x, sm); break;
+    case 6: fine_synthesis<T, S, 6, LV>(A, x, sm); break;
+    default: fine_synthesis<T, S, 8, LV>(A, x, sm); break;
     }
 }
 
 // A2_k: the finest synthesis level, tiled over all CTAs: nodal = W^{-1} p_k.
-template <typename T, typename S>
+// A2b_k (LV = 1), before it: the level before the finest.
+template <int LV = 0, typename T, typename S>
 __device__ __forceinline__ void phase_A2(const Args<T, S> &A, const Basis &b, int k, T *sm)
 {
-    phase_fine_synth(A, newP(A, b, k), sm);
+    phase_fine_synth<LV>(A, newP(A, b, k), sm);
 }
 
-// D1_k: the finest analysis level of u, tiled over all CTAs.
-template <typename T, typename S>
+// D1_k: the finest analysis level of u, tiled over all CTAs.  D1b_k (LV = 1),
+// after it: the next level.
+template <int LV = 0, typename T, typename S>
 __device__ __forceinline__ void phase_D1(const Args<T, S> &A, T *sm)
 {
-    if (!split_levels(A)) return;
+    if (!split_levels(A) || split_depth(A.geo) <= LV) return;
     switch (A.geo.n_taps) {
-    case 2: fine_analysis<T, S, 2>(A, sm); break;
-    case 4: fine_analysis<T, S, 4>(A, sm); break;
-    case 6: fine_analysis<T, S, 6>(A, sm); break;
-    default: fine_analysis<T, S, 8>(A, sm); break;
+    case 2: fine_analysis<T, S, 2, LV>(A, sm); break;
+    case 4: fine_analysis<T, S, 4, LV>(A, sm); break;
+    case 6: fine_analysis<T, S, 6, LV>(A, sm); break;
+    default: fine_analysis<T, S, 8, LV>(A, sm); break;
     }
 }
 
@@ -799,8 +839,8 @@ __device__ __forceinline__ void analysis_update(const Args<T, S> &A, T *buf, Upd
     // detail coefficients (their wq from D1_k)
     if (split_levels(A)) {
         if (A.vrank() < G.L) {
-            const int l = A.vrank(), n = G.lay_n[l], h = n >> 1, lgh = G.lay_lg[l] - 1, nv = h * h / W;
-            const T *ll = A.ll + G.ll_off[l];
+            const int d = split_depth(G), l = A.vrank(), h = G.lay_n[l] >> d, lgh = G.lay_lg[l] - d, nv = h * h / W;
+            const T *ll = ll_block(A, l, d);
 #pragma unroll 4
             for (int v = threadIdx.x; v < nv; v += blockDim.x) {
                 T x[W];
@@ -810,7 +850,7 @@ __device__ __forceinline__ void analysis_update(const Args<T, S> &A, T *buf, Upd
                 for (int i = 0; i < W; i++) buf[s0 + i] = x[i];
             }
             __syncthreads();
-            fdwt2<T>(buf, G.pingpong ? buf + h * (h + 1) : buf, lgh, G.lay_J[l] - 1, G);
+            fdwt2<T>(buf, G.pingpong ? buf + h * (h + 1) : buf, lgh, G.lay_J[l] - d, G);
             const T sc = G.inv_delta[l];
             for_block_vectors(G, l, [&](long e, int be) {
                 T wq[W];
@@ -1058,24 +1098,25 @@ __device__ __forceinline__ void phase_rhs_update(const Args<T, S> &A, const Basi
 //        z = J^{-1} r and the partial sums of the next step (replacing D2E_k's)
 // Iteration k+1 then takes its scalars from the true residual.
 // ---------------------------------------------------------------------------
-template <typename T>
-__device__ __forceinline__ void phase_TU(const Args<T, T> &A, T *buf)
+// The coarser synthesis levels of vector x (whole form: every level, to nodal).
+template <typename T, typename S>
+__device__ __forceinline__ void phase_coarse_synth(const Args<T, S> &A, const T *x0, T *buf)
 {
     constexpr int W = VW<T>::W;
     const Geo<T> &G = A.geo;
     if (split_levels(A)) {
         if (A.vrank() < G.L) {
-            const int l = A.vrank(), h = G.lay_n[l] >> 1, lgh = G.lay_lg[l] - 1;
+            const int d = split_depth(G), l = A.vrank(), h = G.lay_n[l] >> d, lgh = G.lay_lg[l] - d;
             for_block_vectors(G, l, [&](long e, int be) {
                 T x[W];
-                vld_cg(A.c + e, x);
+                vld_cg(x0 + e, x);
                 const int s0 = spad(be, lgh);
 #pragma unroll
                 for (int i = 0; i < W; i++) buf[s0 + i] = x[i];
             });
             __syncthreads();
-            idwt2<T>(buf, G.pingpong ? buf + h * (h + 1) : buf, lgh, G.lay_J[l] - 1, G);
-            T *ll = A.ll + G.ll_off[l];
+            idwt2<T>(buf, G.pingpong ? buf + h * (h + 1) : buf, lgh, G.lay_J[l] - d, G);
+            T *ll = ll_block(A, l, d);
             for (int v = threadIdx.x; v < h * h / W; v += blockDim.x) {
                 const int be = v * W, s0 = spad(be, lgh);
                 T x[W];
@@ -1086,8 +1127,14 @@ __device__ __forceinline__ void phase_TU(const Args<T, T> &A, T *buf)
             __syncthreads();
         }
     } else {
-        layer_idwt<T, T>(A, buf, [&](long e, T (&x)[W]) { vld_cg(A.c + e, x); });
+        layer_idwt<T, S>(A, buf, [&](long e, T (&x)[W]) { vld_cg(x0 + e, x); });
     }
+}
+
+template <typename T>
+__device__ __forceinline__ void phase_TU(const Args<T, T> &A, T *buf)
+{
+    phase_coarse_synth(A, A.c, buf);
 }
 
 template <typename T>
