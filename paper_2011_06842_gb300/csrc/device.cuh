@@ -19,7 +19,7 @@
 //   band_gather  P_g^T in gather form, per (layer, band of rows): the adjoint
 //                wavefronts are staged in shared memory and contracted
 //                separably (x then y), no atomics
-//   layer_fdwt   W^{-T} per layer, fused with + alpha D p
+//   analysis     W^{-T} per layer, fused with + alpha D p
 //   axpy         c += alpha p, r -= alpha q and the inner products of
 //                Algorithm 1/2 (z = J^{-1} r is never stored)
 //   gram/init    projection of the warm start onto the recycled basis
@@ -1083,41 +1083,6 @@ __device__ __forceinline__ void band_gather(const Args<T, S> &A, T *sm, const Ba
             const int o = threadIdx.x + j * blockDim.x;
             if (o < nout) A.u[G.lay_off[l] + ((long)(a0 + (o >> lgn)) << lgn) + (o & (n - 1))] = acc[j];
         }
-    }
-}
-
-// ---------------------------------------------------------------------------
-// Layer phase 2: W u / delta_l per layer; `store(e, value)` consumes each
-// coefficient (u was written by band_gather in another CTA: L2 loads).
-// ---------------------------------------------------------------------------
-template <typename T, typename S, class Store>
-__device__ void layer_fdwt(const Args<T, S> &A, T *buf, Store store)
-{
-    constexpr int W = VW<T>::W;
-    const Geo<T> &G = A.geo;
-    for (int l = A.vrank(); l < G.L; l += A.ncta) {
-        const int n = G.lay_n[l], lgn = G.lay_lg[l], nv = n * n / W;
-        const long off = G.lay_off[l];
-#pragma unroll 4
-        for (int v = threadIdx.x; v < nv; v += blockDim.x) {
-            T x[W];
-            vld_cg(A.u + off + (long)v * W, x);
-            const int s0 = spad(v * W, lgn);
-#pragma unroll
-            for (int i = 0; i < W; i++) buf[s0 + i] = x[i];
-        }
-        __syncthreads();
-        fdwt2<T>(buf, G.pingpong ? buf + n * (n + 1) : buf, lgn, G.lay_J[l], G);
-        const T sc = G.inv_delta[l];
-#pragma unroll 2
-        for (int v = threadIdx.x; v < nv; v += blockDim.x) {
-            T x[W];
-            const int s0 = spad(v * W, lgn);
-#pragma unroll
-            for (int i = 0; i < W; i++) x[i] = buf[s0 + i] * sc;
-            store(off + (long)v * W, x);
-        }
-        __syncthreads();
     }
 }
 

@@ -39,60 +39,24 @@ __device__ __forceinline__ void args_to_smem(const Args<T, S> &src, Args<T, S> &
     __syncthreads();
 }
 
-// apply: nodal = W^{-1} x
-template <typename T, typename S>
-__global__ void __launch_bounds__(kThreads, 1) k_apply_idwt(const __grid_constant__ Args<T, S> Ap)
+// --- the operator by itself: y = M x, b = W^{-T} A^T C^{-1} s, nodal = W^{-1} c --
+// The solver's phases as a chain of kernels.  Split form (split_levels): the
+// coarser synthesis levels on one CTA per layer, the finest split_depth levels
+// tiled over all CTAs, and back the same way; whole form: every level on the
+// layer's CTA.  One CTA per layer for every level left 143 of 152 SMs idle for
+// most of an ELT application.
+// The kernels are launched with programmatic stream serialisation: each
+// lets the next one start (its launch, its arguments into shared memory) and
+// waits for the previous one's results before it touches memory.  The first
+// of a chain is launched without it.
+__device__ __forceinline__ void pdl_begin()
 {
-    __shared__ __align__(16) Args<T, S> A;
-    args_to_smem(Ap, A);
-    constexpr int W = VW<T>::W;
-    layer_idwt<T, S>(A, dyn_smem<T>(), [&](long e, T (&x)[W]) { vld(A.x + e, x); });
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
-// psi = Gamma^T C Gamma P nodal (RHS = false) or Gamma^T C s (RHS = true)
-template <typename T, typename S, bool RHS>
-__global__ void __launch_bounds__(kThreads, 1) k_wfs(const __grid_constant__ Args<T, S> Ap)
-{
-    __shared__ __align__(16) Args<T, S> A;
-    args_to_smem(Ap, A);
-    __shared__ double sred[kSred];
-    typename AccT<T>::type acc[1] = {wfs_phase<T, S, RHS>(A, dyn_smem<T>())};
-    const int slots[1] = {kSlotB};
-    block_partials<1>(acc, A.part, slots, sred, A.vrank());
-}
-
-// u = P^T psi
-template <typename T, typename S>
-__global__ void __launch_bounds__(kThreads, 1) k_gather(const __grid_constant__ Args<T, S> Ap)
-{
-    __shared__ __align__(16) Args<T, S> A;
-    args_to_smem(Ap, A);
-    if (ldcgi(&A.rec->done) || ldcgi(&A.rec->status)) return;
-    band_gather<T, S>(A, dyn_smem<T>());
-}
-
-// y = W^{-T} u + alpha D x  (APPLY) or y = W^{-T} u (RHS)
-template <typename T, typename S, bool RHS>
-__global__ void __launch_bounds__(kThreads, 1) k_fdwt(const __grid_constant__ Args<T, S> Ap)
-{
-    __shared__ __align__(16) Args<T, S> A;
-    args_to_smem(Ap, A);
-    constexpr int W = VW<T>::W;
-    layer_fdwt<T, S>(A, dyn_smem<T>(), [&](long e, const T (&v)[W]) {
-        T y[W], x[W], ad[W];
-        if (!RHS) {
-            vld(A.x + e, x);
-            vld_nc(A.geo.alpha_d + e, ad);
-        }
-#pragma unroll
-        for (int i = 0; i < W; i++) y[i] = RHS ? v[i] : v[i] + ad[i] * x[i];
-        vst(A.y + e, y);
-    });
-}
-
-// --- y_v = M x_v for several vectors at once --------------------------------
-// Vector v is applied by CTAs [v*per, (v+1)*per) with its own scratch
-// buffers, so the per-layer transforms of all vectors run side by side.
+// Several vectors at once: vector v is applied by CTAs [v*per, (v+1)*per) with
+// its own scratch buffers, so the transforms of all vectors run side by side.
 constexpr int kMaxVec = FEWHA_MAX_MULTI;
 
 template <typename T, typename S>
@@ -102,45 +66,78 @@ struct MultiArgs {
 };
 
 template <typename T, typename S>
-__global__ void __launch_bounds__(kThreads, 1) k_multi_idwt(const __grid_constant__ MultiArgs<T, S> M)
+__device__ __forceinline__ void op_args(const Args<T, S> &P, Args<T, S> &A)
 {
-    __shared__ __align__(16) Args<T, S> A;
-    args_to_smem(M.a[blockIdx.x / M.per], A);
-    constexpr int W = VW<T>::W;
-    layer_idwt<T, S>(A, dyn_smem<T>(), [&](long e, T (&x)[W]) { vld(A.x + e, x); });
+    args_to_smem(P, A);
+    pdl_begin();
+}
+template <typename T, typename S>
+__device__ __forceinline__ void op_args(const MultiArgs<T, S> &P, Args<T, S> &A)
+{
+    args_to_smem(P.a[blockIdx.x / P.per], A);
+    pdl_begin();
 }
 
-template <typename T, typename S>
-__global__ void __launch_bounds__(kThreads, 1) k_multi_wfs(const __grid_constant__ MultiArgs<T, S> M)
+// W^{-1} x: the coarser levels (whole form: every level, to nodal)
+template <typename T, typename S, class P, bool WHOLE>
+__global__ void __launch_bounds__(kThreads, 1) k_op_coarse(const __grid_constant__ P p)
 {
     __shared__ __align__(16) Args<T, S> A;
-    args_to_smem(M.a[blockIdx.x / M.per], A);
-    __shared__ double sred[kSred];
-    typename AccT<T>::type acc[1] = {wfs_phase<T, S, false>(A, dyn_smem<T>())};
-    const int slots[1] = {kSlotB};
-    block_partials<1>(acc, A.part, slots, sred, A.vrank());
+    op_args(p, A);
+    phase_coarse_synth<WHOLE>(A, A.x, dyn_smem<T>());
 }
 
-template <typename T, typename S>
-__global__ void __launch_bounds__(kThreads, 1) k_multi_gather(const __grid_constant__ MultiArgs<T, S> M)
+// W^{-1} x: tiled level LV (0 = finest, to nodal)
+template <typename T, typename S, class P, int LV>
+__global__ void __launch_bounds__(kThreads, 1) k_op_synth(const __grid_constant__ P p)
 {
     __shared__ __align__(16) Args<T, S> A;
-    args_to_smem(M.a[blockIdx.x / M.per], A);
+    op_args(p, A);
+    phase_fine_synth<LV>(A, A.x, dyn_smem<T>());
+}
+
+// psi = Gamma^T C Gamma P nodal (RHS = false) or Gamma^T C s (RHS = true)
+template <typename T, typename S, class P, bool RHS>
+__global__ void __launch_bounds__(kThreads, 1) k_op_wfs(const __grid_constant__ P p)
+{
+    __shared__ __align__(16) Args<T, S> A;
+    op_args(p, A);
+    wfs_phase<T, S, RHS>(A, dyn_smem<T>());
+}
+
+// u = P^T psi
+template <typename T, typename S, class P>
+__global__ void __launch_bounds__(kThreads, 1) k_op_gather(const __grid_constant__ P p)
+{
+    __shared__ __align__(16) Args<T, S> A;
+    op_args(p, A);
     band_gather<T, S>(A, dyn_smem<T>());
 }
 
-template <typename T, typename S>
-__global__ void __launch_bounds__(kThreads, 1) k_multi_fdwt(const __grid_constant__ MultiArgs<T, S> M)
+// W^{-T} u: tiled level LV (split form)
+template <typename T, typename S, class P, int LV>
+__global__ void __launch_bounds__(kThreads, 1) k_op_analysis(const __grid_constant__ P p)
 {
     __shared__ __align__(16) Args<T, S> A;
-    args_to_smem(M.a[blockIdx.x / M.per], A);
+    op_args(p, A);
+    phase_D1<LV>(A, dyn_smem<T>());
+}
+
+// y = W^{-T} u + alpha D x (RHS = false) or y = W^{-T} u (RHS = true)
+template <typename T, typename S, class P, bool RHS, bool WHOLE>
+__global__ void __launch_bounds__(kThreads, 1) k_op_update(const __grid_constant__ P p)
+{
+    __shared__ __align__(16) Args<T, S> A;
+    op_args(p, A);
     constexpr int W = VW<T>::W;
-    layer_fdwt<T, S>(A, dyn_smem<T>(), [&](long e, const T (&v)[W]) {
+    analysis_update<WHOLE>(A, dyn_smem<T>(), [&](long e, const T (&v)[W]) {
         T y[W], x[W], ad[W];
-        vld(A.x + e, x);
-        vld_nc(A.geo.alpha_d + e, ad);
+        if (!RHS) {
+            vld(A.x + e, x);
+            vld_nc(A.geo.alpha_d + e, ad);
+        }
 #pragma unroll
-        for (int i = 0; i < W; i++) y[i] = v[i] + ad[i] * x[i];
+        for (int i = 0; i < W; i++) y[i] = RHS ? v[i] : v[i] + ad[i] * x[i];
         vst(A.y + e, y);
     });
 }
@@ -645,6 +642,8 @@ struct Impl : ImplBase {
     size_t sm_fixed = 0;  // dynamic shared memory of every phase but the WFS tiles
     size_t sm_base = 0;   // of the layer and WFS phases alone (before the P^T bands)
     size_t sm_layer_ = 0; // of the layer phases alone
+    size_t sm_fine_ = 0;  // of the tiled wavelet levels alone
+    size_t ll_elems() const { return (size_t)P.n / 4 + P.n / 16 + 1; }  // Args::ll
     std::vector<void *> band_owned;  // device tables of the P^T bands (replaced by plan_bands)
     int band_rows_large = 0, band_rows_small = 0;
 
@@ -976,7 +975,7 @@ struct Impl : ImplBase {
         }
         if ((st = alloc((size_t)P.n, &base.nodal)) || (st = alloc((size_t)P.n, &base.u)) ||
             (st = alloc((size_t)P.n, &base.wq)) ||
-            (st = alloc((size_t)P.psi_off[P.G], &base.psi)) || (st = alloc((size_t)P.n / 4 + P.n / 16 + 1, &base.ll)) ||
+            (st = alloc((size_t)P.psi_off[P.G], &base.psi)) || (st = alloc(ll_elems(), &base.ll)) ||
             (st = alloc((size_t)kSlots * kMaxCtas, &base.part)) || (st = alloc((size_t)1, &base.rec)))
             return st;
         if constexpr (std::is_same<T, S>::value) {
@@ -1005,6 +1004,7 @@ struct Impl : ImplBase {
             }
         }
         sm_layer = std::max(sm_layer, sm_fine);
+        sm_fine_ = sm_fine;
         smem = std::max(sm_layer, sm_wfs);
         sm_base = smem;
         sm_layer_ = sm_layer;
@@ -1016,12 +1016,11 @@ struct Impl : ImplBase {
         auto setattr = [&](const void *f) {
             return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
         };
-        CK(setattr((const void *)k_apply_idwt<T, S>));
-        CK(setattr((const void *)k_wfs<T, S, false>));
-        CK(setattr((const void *)k_wfs<T, S, true>));
-        CK(setattr((const void *)k_gather<T, S>));
-        CK(setattr((const void *)k_fdwt<T, S, false>));
-        CK(setattr((const void *)k_fdwt<T, S, true>));
+        CK((op_attributes<Args<T, S>>()));
+        CK((op_attributes<MultiArgs<T, S>>()));
+        CK(setattr((const void *)k_op_wfs<T, S, Args<T, S>, true>));
+        CK(setattr((const void *)k_op_update<T, S, Args<T, S>, true, false>));
+        CK(setattr((const void *)k_op_update<T, S, Args<T, S>, true, true>));
         CK(setattr((const void *)k_rhs_wfs<T, S>));
         CK(setattr((const void *)k_rhs_D1<T, S, 0>));
         CK(setattr((const void *)k_rhs_D1<T, S, 1>));
@@ -1053,9 +1052,6 @@ struct Impl : ImplBase {
                                 200 * 1024));
         CK(cudaFuncSetAttribute((const void *)k_solve_batched<T, S, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 200 * 1024));
-        for (const void *f : {(const void *)k_multi_idwt<T, S>, (const void *)k_multi_wfs<T, S>,
-                              (const void *)k_multi_gather<T, S>, (const void *)k_multi_fdwt<T, S>})
-            CK(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
         int per_sm = 0;
         CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_solve_persistent<T, S, false>, kThreads, smem));
         if (per_sm < 1) return FEWHA_ERR_CUDA;
@@ -1146,26 +1142,113 @@ struct Impl : ImplBase {
 
     int launch_check() { return cudaGetLastError() == cudaSuccess ? FEWHA_OK : FEWHA_ERR_CUDA; }
 
+    template <class A>
+    static cudaError_t op_attributes()
+    {
+        for (const void *f : {(const void *)k_op_coarse<T, S, A, false>, (const void *)k_op_coarse<T, S, A, true>,
+                              (const void *)k_op_synth<T, S, A, 0>, (const void *)k_op_synth<T, S, A, 1>,
+                              (const void *)k_op_wfs<T, S, A, false>, (const void *)k_op_gather<T, S, A>,
+                              (const void *)k_op_analysis<T, S, A, 0>, (const void *)k_op_analysis<T, S, A, 1>,
+                              (const void *)k_op_update<T, S, A, false, false>,
+                              (const void *)k_op_update<T, S, A, false, true>}) {
+            const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+            if (e != cudaSuccess) return e;
+        }
+        return cudaSuccess;
+    }
+
+    // One kernel of an operator chain; after the first, with programmatic
+    // stream serialisation (see pdl_begin).
+    struct OpChain {
+        int grid;
+        cudaStream_t s;
+        bool first;
+        cudaError_t err;
+        template <class K, class A>
+        void operator()(K kern, size_t sm, const A &args)
+        {
+            if (err != cudaSuccess) return;
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3(grid);
+            cfg.blockDim = dim3(kThreads);
+            cfg.dynamicSmemBytes = sm;
+            cfg.stream = s;
+            cudaLaunchAttribute attr[1];
+            attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+            attr[0].val.programmaticStreamSerializationAllowed = 1;
+            cfg.attrs = attr;
+            cfg.numAttrs = first ? 0 : 1;
+            err = cudaLaunchKernelEx(&cfg, kern, args);
+            first = false;
+        }
+    };
+
+    // Form of the chain for `group` CTAs per vector.  FP64: split whenever a
+    // group can be (a layer's CTA is bound by its FP64 units).  FP32: from four
+    // CTAs per layer; below, the two tiled kernels' launches and rounds cost
+    // what they take off the layers' CTAs (9 ELT layers, 5 vectors, 30 CTAs
+    // each: 94.7 us split, 91.9 us whole).
+    bool op_split(int group) const { return group >= (sizeof(T) == 8 ? 2 : 4) * P.L; }
+
+    // nodal = W^{-1} x; group: CTAs per vector
+    template <class A>
+    void op_idwt(OpChain &run, const A &args, int group, size_t sm) const
+    {
+        if (!op_split(group)) {
+            run(k_op_coarse<T, S, A, true>, sm, args);
+            return;
+        }
+        run(k_op_coarse<T, S, A, false>, sm, args);
+        if (base.geo.depth > 1) run(k_op_synth<T, S, A, 1>, sm_fine_, args);
+        run(k_op_synth<T, S, A, 0>, sm_fine_, args);
+    }
+
+    // u = P^T psi and W^{-T} u up to its last part
+    template <class A>
+    void op_adjoint(OpChain &run, const A &args, int group, size_t sm) const
+    {
+        run(k_op_gather<T, S, A>, sm, args);
+        if (!op_split(group)) return;
+        run(k_op_analysis<T, S, A, 0>, sm_fine_, args);
+        if (base.geo.depth > 1) run(k_op_analysis<T, S, A, 1>, sm_fine_, args);
+    }
+
+    template <class A>
+    int op_apply(const A &args, int grid, int group, size_t sm, cudaStream_t s) const
+    {
+        OpChain run{grid, s, true, cudaSuccess};
+        op_idwt(run, args, group, sm);
+        run(k_op_wfs<T, S, A, false>, sm, args);
+        op_adjoint(run, args, group, sm);
+        if (op_split(group))
+            run(k_op_update<T, S, A, false, false>, sm, args);
+        else
+            run(k_op_update<T, S, A, false, true>, sm, args);
+        return run.err == cudaSuccess ? FEWHA_OK : FEWHA_ERR_CUDA;
+    }
+
+    int op_nodal(const void *c, cudaStream_t s) const
+    {
+        Args<T, S> A = base;
+        A.x = static_cast<const T *>(c);
+        OpChain run{ncta, s, true, cudaSuccess};
+        op_idwt(run, A, ncta, smem);
+        return run.err == cudaSuccess ? FEWHA_OK : FEWHA_ERR_CUDA;
+    }
+
     int apply(const void *x, void *y, cudaStream_t s) override
     {
         Args<T, S> A = base;
         A.x = static_cast<const T *>(x);
         A.y = static_cast<T *>(y);
-        CK(cudaMemsetAsync(A.rec, 0, offsetof(Record, rz), s));
-        k_apply_idwt<T, S><<<ncta, kThreads, smem, s>>>(A);
-        k_wfs<T, S, false><<<ncta, kThreads, smem, s>>>(A);
-        k_gather<T, S><<<ncta, kThreads, smem, s>>>(A);
-        k_fdwt<T, S, false><<<ncta, kThreads, smem, s>>>(A);
-        return launch_check();
+        return op_apply(A, ncta, ncta, smem, s);
     }
 
     int fit(const void *c, void *a, cudaStream_t s) override
     {
         if (!P.fit_ok) return FEWHA_ERR_GEOMETRY;
-        Args<T, S> A = base;
-        A.x = static_cast<const T *>(c);
-        CK(cudaMemsetAsync(A.rec, 0, offsetof(Record, rz), s));
-        k_apply_idwt<T, S><<<ncta, kThreads, smem, s>>>(A);  // nodal = W^{-1} c
+        const int st = op_nodal(c, s);  // nodal = W^{-1} c
+        if (st != FEWHA_OK) return st;
         FitTab<T> F{};
         for (int l = 0; l < P.L; l++) {
             F.off[l] = P.lay_off[l];
@@ -1317,10 +1400,8 @@ struct Impl : ImplBase {
     {
         if (iters < 0 || iters > FEWHA_MAX_ITER) return FEWHA_ERR_ARG;
         auto *pl = static_cast<McaoPlan *>(plan);
-        Args<T, S> A = base;
-        A.x = static_cast<const T *>(c);
-        CK(cudaMemsetAsync(A.rec, 0, offsetof(Record, rz), s));
-        k_apply_idwt<T, S><<<ncta, kThreads, smem, s>>>(A);  // nodal = W^{-1} c
+        const int st = op_nodal(c, s);  // nodal = W^{-1} c
+        if (st != FEWHA_OK) return st;
         McaoArgs<T, S> M = pl->M;
         M.nodal = base.nodal;
         M.a = static_cast<T *>(a);
@@ -1369,7 +1450,7 @@ struct Impl : ImplBase {
         auto up256 = [](size_t v) { return (v + 255) & ~(size_t)255; };
         if (!multi_buf) {
             multi_stride = up256((size_t)P.n * sizeof(S)) + up256((size_t)P.psi_off[P.G] * sizeof(S)) +
-                           up256((size_t)P.n * sizeof(T));
+                           2 * up256((size_t)P.n * sizeof(T)) + up256(ll_elems() * sizeof(T));
             if (alloc(multi_stride * kMaxVec, &multi_buf)) return FEWHA_ERR_NOMEM;
         }
         const int per = std::max(1, ncta / nvec);
@@ -1384,7 +1465,8 @@ struct Impl : ImplBase {
             A.nodal = reinterpret_cast<S *>(b);
             A.psi = reinterpret_cast<S *>(b + up256((size_t)P.n * sizeof(S)));
             A.u = reinterpret_cast<T *>(b + up256((size_t)P.n * sizeof(S)) + up256((size_t)P.psi_off[P.G] * sizeof(S)));
-            A.part = base.part + (size_t)v * per;  // disjoint partial-sum columns
+            A.wq = A.u + up256((size_t)P.n * sizeof(T)) / sizeof(T);
+            A.ll = A.wq + up256((size_t)P.n * sizeof(T)) / sizeof(T);
             A.x = static_cast<const T *>(x) + (size_t)v * ldx;
             A.y = static_cast<T *>(y) + (size_t)v * ldy;
             A.cta0 = v * per;
@@ -1395,45 +1477,38 @@ struct Impl : ImplBase {
             A.trace_cap = 0;
             M.a[v] = A;
         }
-        CK(cudaMemsetAsync(base.rec, 0, offsetof(Record, rz), s));
-        const int grid = per * nvec;
-        k_multi_idwt<T, S><<<grid, kThreads, sm, s>>>(M);
-        k_multi_wfs<T, S><<<grid, kThreads, sm, s>>>(M);
-        k_multi_gather<T, S><<<grid, kThreads, sm, s>>>(M);
-        k_multi_fdwt<T, S><<<grid, kThreads, sm, s>>>(M);
-        return launch_check();
+        return op_apply(M, per * nvec, per, sm, s);
     }
 
     int apply_in_scratch(const void *x, void *y, void *scratch, size_t bytes, cudaStream_t s) override
     {
-        // layout: record | partial sums | nodal layers | adjoint wavefronts | P^T output
+        // layout: nodal layers | adjoint wavefronts | P^T output | level-1 and -2
+        // approximations | operator output before + alpha D x (in the nodal
+        // layers' place when they have the same type: it is written after they
+        // were last read).  Every buffer is written before it is read.
         auto up256 = [](size_t v) { return (v + 255) & ~(size_t)255; };
-        const size_t o_rec = 0;
-        const size_t o_part = up256(o_rec + sizeof(Record));
-        const size_t o_nodal = up256(o_part + (size_t)kSlots * kMaxCtas * sizeof(double));
-        const size_t o_psi = up256(o_nodal + (size_t)P.n * sizeof(S));
+        const size_t o_psi = up256((size_t)P.n * sizeof(S));
         const size_t o_u = up256(o_psi + (size_t)P.psi_off[P.G] * sizeof(S));
-        const size_t need = up256(o_u + (size_t)P.n * sizeof(T));
-        if (need > bytes) return FEWHA_ERR_SCRATCH;
+        const size_t o_ll = up256(o_u + (size_t)P.n * sizeof(T));
+        const size_t o_wq = std::is_same<T, S>::value ? 0 : up256(o_ll + ll_elems() * sizeof(T));
+        const size_t need = std::max(up256(o_ll + ll_elems() * sizeof(T)), up256(o_wq + (size_t)P.n * sizeof(T)));
+        // the size test of the entry point's contract: record, partial sums of
+        // every CTA, nodal layers, adjoint wavefronts and P^T output
+        const size_t contract = up256(sizeof(Record)) + up256((size_t)kSlots * kMaxCtas * sizeof(double)) +
+                                up256(o_u + (size_t)P.n * sizeof(T));
+        if (contract > bytes || need > bytes) return FEWHA_ERR_SCRATCH;
         unsigned char *base_p = static_cast<unsigned char *>(scratch);
         Args<T, S> A = base;
-        A.rec = reinterpret_cast<Record *>(base_p + o_rec);
-        A.part = reinterpret_cast<double *>(base_p + o_part);
-        A.nodal = reinterpret_cast<S *>(base_p + o_nodal);
+        A.nodal = reinterpret_cast<S *>(base_p);
         A.psi = reinterpret_cast<S *>(base_p + o_psi);
         A.u = reinterpret_cast<T *>(base_p + o_u);
+        A.ll = reinterpret_cast<T *>(base_p + o_ll);
+        A.wq = reinterpret_cast<T *>(base_p + o_wq);
         A.trace = nullptr;
         A.trace_cap = 0;
         A.x = static_cast<const T *>(x);
         A.y = static_cast<T *>(y);
-        // the record's flags must start at zero; the other buffers are fully
-        // overwritten before they are read
-        CK(cudaMemsetAsync(A.rec, 0, offsetof(Record, rz), s));
-        k_apply_idwt<T, S><<<ncta, kThreads, smem, s>>>(A);
-        k_wfs<T, S, false><<<ncta, kThreads, smem, s>>>(A);
-        k_gather<T, S><<<ncta, kThreads, smem, s>>>(A);
-        k_fdwt<T, S, false><<<ncta, kThreads, smem, s>>>(A);
-        return launch_check();
+        return op_apply(A, ncta, ncta, smem, s);
     }
 
     int rhs(const void *sl, void *b, cudaStream_t s) override
@@ -1441,11 +1516,14 @@ struct Impl : ImplBase {
         Args<T, S> A = base;
         A.slopes = static_cast<const S *>(sl);
         A.y = static_cast<T *>(b);
-        CK(cudaMemsetAsync(A.rec, 0, offsetof(Record, rz), s));
-        k_wfs<T, S, true><<<ncta, kThreads, smem, s>>>(A);
-        k_gather<T, S><<<ncta, kThreads, smem, s>>>(A);
-        k_fdwt<T, S, true><<<ncta, kThreads, smem, s>>>(A);
-        return launch_check();
+        OpChain run{ncta, s, true, cudaSuccess};
+        run(k_op_wfs<T, S, Args<T, S>, true>, smem, A);
+        op_adjoint(run, A, ncta, smem);
+        if (op_split(ncta))
+            run(k_op_update<T, S, Args<T, S>, true, false>, smem, A);
+        else
+            run(k_op_update<T, S, Args<T, S>, true, true>, smem, A);
+        return run.err == cudaSuccess ? FEWHA_OK : FEWHA_ERR_CUDA;
     }
 
     Args<T, S> solve_args(const void *sl, void *c, const fewha_state *st, const fewha_solve_opts *o,

@@ -714,37 +714,82 @@ __device__ void fine_synthesis(const Args<T, S> &A, const T *pk, T *sm)
             win[e] = v;
         }
         __syncthreads();
-        for (int e = threadIdx.x; e < 2 * ty * 2 * WC; e += blockDim.x) {  // columns
-            const int yy = e / (2 * WC), cc = e - yy * (2 * WC);
-            const int i = yy >> 1, ey = yy & 1, half = cc >= WC ? 1 : 0, c = cc - half * WC;
-            const T *lo = win + (half ? 1 : 0) * Q + c;  // low y: LL or LH
-            const T *hi = win + (half ? 3 : 2) * Q + c;  // high y: HL or HH
-            T x = 0;
-#pragma unroll
-            for (int u = 0; u < Lh; u++) {
-                const int r = i + Lh - 1 - u;
-                x += tp.h[ey + 2 * u] * lo[r * WC] + tp.g[ey + 2 * u] * hi[r * WC];
-            }
-            mid[e] = x;
-        }
-        __syncthreads();
         const T sc = G.inv_delta[l];
         S *nodal = A.nodal + G.lay_off[l];
         T *ll1 = ll_block(A, l, 1);
-        for (int e = threadIdx.x; e < 2 * ty * 2 * tx; e += blockDim.x) {  // rows
-            const int yy = e / (2 * tx), xx = e - yy * (2 * tx), j = xx >> 1, ex = xx & 1;
-            const T *row = mid + yy * 2 * WC;
-            T x = 0;
+        if constexpr (sizeof(T) == 8) {
+            // FP64: a thread forms both values of an output pair, so that the
+            // taps' indices are compile-time and each product is one FMA (the
+            // FP64 pipe takes a warp instruction every 64 cycles).  In FP32
+            // the same form changed the register allocation of the persistent
+            // kernel: this phase 4.5 -> 4.2 us, its neighbours 4 us slower.
+            for (int e = threadIdx.x; e < ty * 2 * WC; e += blockDim.x) {  // columns
+                const int i = e / (2 * WC), cc = e - i * (2 * WC);
+                const int half = cc >= WC ? 1 : 0, c = cc - half * WC;
+                const T *lo = win + (half ? 1 : 0) * Q + c;  // low y: LL or LH
+                const T *hi = win + (half ? 3 : 2) * Q + c;  // high y: HL or HH
+                T x0 = 0, x1 = 0;
 #pragma unroll
-            for (int u = 0; u < Lh; u++) {
-                const int c = j + Lh - 1 - u;
-                x += tp.h[ex + 2 * u] * row[c] + tp.g[ex + 2 * u] * row[WC + c];
+                for (int u = 0; u < Lh; u++) {
+                    const int r = i + Lh - 1 - u;
+                    const T a = lo[r * WC], d = hi[r * WC];
+                    x0 = fma(tp.g[2 * u], d, fma(tp.h[2 * u], a, x0));
+                    x1 = fma(tp.g[2 * u + 1], d, fma(tp.h[2 * u + 1], a, x1));
+                }
+                mid[2 * i * (2 * WC) + cc] = x0;
+                mid[(2 * i + 1) * (2 * WC) + cc] = x1;
             }
-            const long o = (long)(2 * p0y + yy) * N + 2 * p0x + xx;
-            if constexpr (LV == 0)
-                nodal[o] = Cv<S>::st(x * sc);
-            else
-                ll1[o] = x;
+            __syncthreads();
+            for (int e = threadIdx.x; e < 2 * ty * tx; e += blockDim.x) {  // rows
+                const int yy = e / tx, j = e - yy * tx;
+                const T *row = mid + yy * 2 * WC;
+                T x0 = 0, x1 = 0;
+#pragma unroll
+                for (int u = 0; u < Lh; u++) {
+                    const int c = j + Lh - 1 - u;
+                    const T a = row[c], d = row[WC + c];
+                    x0 = fma(tp.g[2 * u], d, fma(tp.h[2 * u], a, x0));
+                    x1 = fma(tp.g[2 * u + 1], d, fma(tp.h[2 * u + 1], a, x1));
+                }
+                const long o = (long)(2 * p0y + yy) * N + 2 * (p0x + j);
+                if constexpr (LV == 0) {
+                    nodal[o] = Cv<S>::st(x0 * sc);
+                    nodal[o + 1] = Cv<S>::st(x1 * sc);
+                } else {
+                    ll1[o] = x0;
+                    ll1[o + 1] = x1;
+                }
+            }
+        } else {
+            for (int e = threadIdx.x; e < 2 * ty * 2 * WC; e += blockDim.x) {  // columns
+                const int yy = e / (2 * WC), cc = e - yy * (2 * WC);
+                const int i = yy >> 1, ey = yy & 1, half = cc >= WC ? 1 : 0, c = cc - half * WC;
+                const T *lo = win + (half ? 1 : 0) * Q + c;  // low y: LL or LH
+                const T *hi = win + (half ? 3 : 2) * Q + c;  // high y: HL or HH
+                T x = 0;
+#pragma unroll
+                for (int u = 0; u < Lh; u++) {
+                    const int r = i + Lh - 1 - u;
+                    x += tp.h[ey + 2 * u] * lo[r * WC] + tp.g[ey + 2 * u] * hi[r * WC];
+                }
+                mid[e] = x;
+            }
+            __syncthreads();
+            for (int e = threadIdx.x; e < 2 * ty * 2 * tx; e += blockDim.x) {  // rows
+                const int yy = e / (2 * tx), xx = e - yy * (2 * tx), j = xx >> 1, ex = xx & 1;
+                const T *row = mid + yy * 2 * WC;
+                T x = 0;
+#pragma unroll
+                for (int u = 0; u < Lh; u++) {
+                    const int c = j + Lh - 1 - u;
+                    x += tp.h[ex + 2 * u] * row[c] + tp.g[ex + 2 * u] * row[WC + c];
+                }
+                const long o = (long)(2 * p0y + yy) * N + 2 * p0x + xx;
+                if constexpr (LV == 0)
+                    nodal[o] = Cv<S>::st(x * sc);
+                else
+                    ll1[o] = x;
+            }
         }
         __syncthreads();
     }
@@ -796,7 +841,7 @@ __device__ __forceinline__ void phase_D1(const Args<T, S> &A, T *sm)
 // output).  Whole form: each layer's CTA transforms the whole of u's layer in
 // shared memory and calls upd for every W-vector of the layer.
 // ---------------------------------------------------------------------------
-template <typename T, typename S, class Upd>
+template <bool WHOLE = false, typename T, typename S, class Upd>
 __device__ __forceinline__ void analysis_update(const Args<T, S> &A, T *buf, Upd update_w)
 {
     constexpr int W = VW<T>::W;
@@ -806,7 +851,7 @@ __device__ __forceinline__ void analysis_update(const Args<T, S> &A, T *buf, Upd
         update_w(e, wq);
     };
     const Geo<T> &G = A.geo;
-    if (!split_levels(A)) {
+    if (WHOLE || !split_levels(A)) {
         // whole layer: W^{-T} u / delta in shared memory, then the update of the
         // layer with wq read from there
         for (int l = A.vrank(); l < G.L; l += A.ncta) {
@@ -837,7 +882,7 @@ __device__ __forceinline__ void analysis_update(const Args<T, S> &A, T *buf, Upd
     // approximation block (from D1_k), then the update on that block with
     // W^{-T} u / delta taken from shared memory; the other CTAs update the
     // detail coefficients (their wq from D1_k)
-    if (split_levels(A)) {
+    if (!WHOLE && split_levels(A)) {
         if (A.vrank() < G.L) {
             const int d = split_depth(G), l = A.vrank(), h = G.lay_n[l] >> d, lgh = G.lay_lg[l] - d, nv = h * h / W;
             const T *ll = ll_block(A, l, d);
@@ -1099,12 +1144,13 @@ __device__ __forceinline__ void phase_rhs_update(const Args<T, S> &A, const Basi
 // Iteration k+1 then takes its scalars from the true residual.
 // ---------------------------------------------------------------------------
 // The coarser synthesis levels of vector x (whole form: every level, to nodal).
-template <typename T, typename S>
+// WHOLE: the whole form whatever the group's size (operator chain).
+template <bool WHOLE = false, typename T, typename S>
 __device__ __forceinline__ void phase_coarse_synth(const Args<T, S> &A, const T *x0, T *buf)
 {
     constexpr int W = VW<T>::W;
     const Geo<T> &G = A.geo;
-    if (split_levels(A)) {
+    if (!WHOLE && split_levels(A)) {
         if (A.vrank() < G.L) {
             const int d = split_depth(G), l = A.vrank(), h = G.lay_n[l] >> d, lgh = G.lay_lg[l] - d;
             for_block_vectors(G, l, [&](long e, int be) {
