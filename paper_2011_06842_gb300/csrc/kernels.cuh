@@ -1369,9 +1369,10 @@ struct Impl : ImplBase {
         };
         const int *c_lk, *c_dk, *c_alo, *c_ahi;
         const T *c_lw, *c_dw;
-        void *r, *p, *q, *y, *part, *rec;
+        void *r, *p, *p2, *q, *y, *part, *rec;
         if (!put_i(lk, &c_lk) || !put_t(lw, &c_lw) || !put_i(dk, &c_dk) || !put_t(dw, &c_dw) ||
             !put_i(alo, &c_alo) || !put_i(ahi, &c_ahi) || !make(na * sizeof(T), &r) || !make(na * sizeof(T), &p) ||
+            !make(na * sizeof(T), &p2) ||
             !make(na * sizeof(T), &q) || !make((size_t)T_ * m * m * sizeof(T), &y) ||
             !make(2 * kMaxCtas * sizeof(double), &part) || !make(sizeof(Record), &rec))
             st = FEWHA_ERR_CUDA;
@@ -1387,6 +1388,7 @@ struct Impl : ImplBase {
         M.ahi = c_ahi;
         M.r = static_cast<T *>(r);
         M.p = static_cast<T *>(p);
+        M.p2 = static_cast<T *>(p2);
         M.q = static_cast<T *>(q);
         M.y = static_cast<T *>(y);
         M.part = static_cast<double *>(part);
