@@ -391,6 +391,16 @@ int fewha_conv3x3_fwd(const float *in, long in_bs, long in_cs, int Cin, const fl
 int fewha_conv3x3_fwd_tc(const float *in, long in_bs, long in_cs, int Cin, const float *w, const float *bias,
                          float *out, long out_bs, long out_cs, int Cout, int B, int H, int W, int relu,
                          int *status_dev, cudaStream_t s);
+/* fewha_convnet_fwd_tc: the network conv(C0 -> 32) ReLU conv(32 -> 32) ReLU
+ *   conv(32 -> C3) in one launch, with the arithmetic of three
+ *   fewha_conv3x3_fwd_tc calls; C0, C3 <= 16.  Image i of group g (count[g]
+ *   images of side[g] x side[g], side <= 128; at most 8 groups; host arrays)
+ *   starts off[g] + i side[g]^2 floats into a channel of in and out; in_cs and
+ *   out_cs are the channel strides.  status_dev as in fewha_conv3x3_fwd_tc. */
+int fewha_convnet_fwd_tc(const float *in, long in_cs, int C0, const float *w1, const float *b1, const float *w2,
+                         const float *b2, const float *w3, const float *b3, float *out, long out_cs, int C3,
+                         int ngroups, const int *count, const int *side, const long *off, int *status_dev,
+                         cudaStream_t s);
 int fewha_conv3x3_bwd_data_relu(const float *gout, long gout_bs, long gout_cs, int Cout, const float *w,
                                 const float *act, float *gin, long gin_bs, long gin_cs, int Cin, int B, int H, int W,
                                 cudaStream_t s);

@@ -289,6 +289,247 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(kTcCols) : "memory");
 }
 
+
+// ---------------------------------------------------------------------------
+// The whole network in one launch (fewha_convnet_fwd_tc): three 3x3
+// convolutions C0 -> 32 -> 32 -> C3 with ReLU after the first two.  A CTA
+// computes R output rows of one image: from R + 6 input rows the R + 4 rows of
+// the first hidden layer and from them the R + 2 of the second, each kept in
+// shared memory as the next convolution's operand (BF16, the rounding a
+// separate convolution applies when it stages its input), so hidden layers
+// neither leave the SM nor are staged four times over (four input rows for two
+// output rows in k_conv3x3_tc).  The images of all sizes share the launch.
+//
+// Latency bound: one CTA per SM, MMAs of 128 x 32 x 16.  Every row of a layer
+// has its own TMEM accumulator and mbarrier, so a layer's epilogue runs behind
+// its MMAs, and the second and third weight images are staged behind the first
+// layer's.
+// ---------------------------------------------------------------------------
+constexpr int kNetC = 32;                  // hidden channels
+constexpr int kNetRows = 8;                // most output rows per CTA
+constexpr int kNetP = 130;                 // staged pixels per (row, channel group): x = -1 .. 128
+constexpr int kNetPlane = kNetP * 16;      // bytes of one (row, channel group)
+constexpr int kNetGroups = 8;              // most image sizes of one launch
+constexpr int kNetW1 = 9 * 2 * 4 * 128, kNetW2 = 9 * 4 * 4 * 128, kNetW3 = 9 * 4 * 2 * 128;  // weight images
+constexpr int kNetCols = 512;              // TMEM columns ((kNetRows + 4) x 32 used)
+constexpr int kNetBars = (kNetRows + 4) + (kNetRows + 2) + kNetRows;
+
+constexpr size_t net_smem(int rows)
+{
+    return (size_t)(2 * rows + 6) * 4 * kNetPlane + kNetW1 + kNetW2 + kNetW3;
+}
+static_assert(net_smem(kNetRows) + 1024 <= 227 * 1024, "shared memory");
+static_assert((kNetRows + 4) * 32 <= kNetCols, "TMEM columns");
+// the input rows (2 channel groups each) fit in the second hidden layer's place
+// for two or more output rows: (R + 6) 2 <= (R + 2) 4
+constexpr int kNetRowsMin = 2;
+
+struct NetGroup {
+    int side, tiles, cta0;  // image side, row tiles per image, first CTA
+    long off;               // of the group's first image in a channel
+};
+struct NetArgs {
+    const float *in, *w1, *b1, *w2, *b2, *w3, *b3;
+    float *out;
+    long in_cs, out_cs;
+    int C0, C3, rows, ngroups;
+    int *status;
+    NetGroup g[kNetGroups];
+};
+
+// w (Cout x Cin x 3 x 3) into the zeroed core-matrix image of NB x 8 output
+// channels and NCG groups of 8 input channels
+template <int NCG, int NB>
+__device__ __forceinline__ void net_weights(const float *__restrict__ w, int Cout, int Cin, unsigned char *Wt)
+{
+    const int nw = Cout * Cin * 9;
+    constexpr int U = 12;  // loads in flight per thread
+    for (int e0 = threadIdx.x; e0 < nw; e0 += U * kTcThreads) {
+        float v[U];
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            const int e = e0 + u * kTcThreads;
+            v[u] = e < nw ? __ldg(w + e) : 0.f;
+        }
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            const int e = e0 + u * kTcThreads;
+            if (e < nw) {
+                const int t = e % 9, cc = e / 9, ci = cc % Cin, co = cc / Cin;
+                unsigned char *row = Wt + (((t * NCG + (ci >> 3)) * NB + (co >> 3)) * 128 + (co & 7) * 16);
+                reinterpret_cast<__nv_bfloat16 *>(row)[ci & 7] = __float2bfloat16_rn(v[u]);
+            }
+        }
+    }
+}
+
+// One layer's MMAs: accumulator i (TMEM columns NC i ..) = sum over taps of row
+// i + ky of `rows` (NCG channel groups); mbarrier i completes with it.  One thread.
+template <int NCG, int N, int NC>
+__device__ __forceinline__ void net_mma(uint32_t rows, uint32_t w, int nrows, uint32_t tmem, uint32_t bars)
+{
+    const uint32_t idesc = instr_desc(N);
+    for (int i = 0; i < nrows; i++) {
+        int acc = 0;
+        for (int t = 0; t < 9; t++) {
+            const int ky = t / 3, kx = t - ky * 3;
+#pragma unroll
+            for (int j = 0; j < NCG; j += 2) {
+                const uint64_t ad =
+                    smem_desc(rows + (uint32_t)(((i + ky) * NCG + j) * kNetPlane + kx * 16), kNetPlane, 128u);
+                const uint64_t bd = smem_desc(w + (uint32_t)((t * NCG + j) * (N / 8) * 128), (N / 8) * 128u, 128u);
+                asm volatile(
+                    "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+                    " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(tmem + (uint32_t)(NC * i)),
+                    "l"(ad), "l"(bd), "r"(idesc), "r"(acc)
+                    : "memory");
+                acc = 1;
+            }
+        }
+        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                         bars + 8u * (uint32_t)i)
+                     : "memory");
+    }
+}
+
+// A hidden layer's epilogue: row i = ReLU(accumulator + bias) of image row
+// yfirst + i as the next operand's row (zero outside the image).  Returns false
+// when a wait ran out.
+__device__ __forceinline__ bool net_hidden(unsigned char *dst, int nrows, int yfirst, int side, const float *bias,
+                                           uint32_t tmem, uint32_t bars)
+{
+    const int warp = threadIdx.x >> 5, x = (warp & 3) * 32 + (threadIdx.x & 31);
+    // the halo pixels x = -1 and x = 128
+    for (int e = threadIdx.x; e < nrows * 4 * 2; e += kTcThreads)
+        *reinterpret_cast<uint4 *>(dst + (size_t)(e >> 1) * kNetPlane + (e & 1) * (kNetP - 1) * 16) =
+            make_uint4(0u, 0u, 0u, 0u);
+    for (int i = warp >> 2; i < nrows; i += kTcThreads / 128) {
+        // the whole warp takes the same way and is converged for the TMEM load
+        if (!__all_sync(0xffffffffu, mbar_wait(bars + 8u * (uint32_t)i, 0))) return false;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        float v[32];
+        tmem_load_row<32>(tmem + 32u * (uint32_t)i + ((uint32_t)((warp & 3) * 32) << 16), v);
+        const bool inside = x < side && yfirst + i >= 0 && yfirst + i < side;
+#pragma unroll
+        for (int g = 0; g < 4; g++) {
+            float r[8];
+#pragma unroll
+            for (int j = 0; j < 8; j++) {
+                const float a = v[8 * g + j] + __ldg(bias + 8 * g + j);
+                r[j] = inside && a > 0.f ? a : 0.f;
+            }
+            *reinterpret_cast<uint4 *>(dst + (size_t)(i * 4 + g) * kNetPlane + (x + 1) * 16) = pack8(r);
+        }
+    }
+    return true;
+}
+
+__global__ void __launch_bounds__(kTcThreads, 1) k_convnet_tc(const __grid_constant__ NetArgs A)
+{
+    extern __shared__ __align__(1024) unsigned char tc_smem[];
+    __shared__ __align__(8) unsigned long long mbar[kNetBars];
+    __shared__ uint32_t tmem_base;
+    const int tid = threadIdx.x, warp = tid >> 5, R = A.rows;
+    int gi = 0;
+    while (gi + 1 < A.ngroups && (int)blockIdx.x >= A.g[gi + 1].cta0) gi++;
+    const NetGroup G = A.g[gi];
+    const int S = G.side, w = (int)blockIdx.x - G.cta0, b = w / G.tiles, y0 = (w - b * G.tiles) * R;
+    const long base = G.off + (long)b * S * S;
+    unsigned char *H1 = tc_smem, *H2 = H1 + (size_t)(R + 4) * 4 * kNetPlane, *W1 = H2 + (size_t)(R + 2) * 4 * kNetPlane;
+    unsigned char *W2 = W1 + kNetW1, *W3 = W2 + kNetW2;
+    unsigned char *X = H2;  // [R + 6][2] planes: dead when the second hidden layer is written
+
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base)),
+                     "r"(kNetCols)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    if (tid < kNetBars) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&mbar[tid])) : "memory");
+    for (int e = tid; e < (kNetW1 + kNetW2 + kNetW3) / 16; e += kTcThreads)
+        reinterpret_cast<uint4 *>(W1)[e] = make_uint4(0u, 0u, 0u, 0u);
+    // input rows y0-3 .. y0+R+2, 8 channels per pixel and group (C0 <= 16)
+    {
+        const int items = (R + 6) * 2 * kNetP;
+        constexpr int U = 4;
+        for (int e0 = tid; e0 < items; e0 += U * kTcThreads) {
+            float v[U][8];
+#pragma unroll
+            for (int u = 0; u < U; u++) {
+                const int e = e0 + u * kTcThreads, pl = e / kNetP, x = e - pl * kNetP - 1, yy = y0 - 3 + (pl >> 1);
+                const bool in = e < items && yy >= 0 && yy < S && x >= 0 && x < S;
+                const float *p = A.in + base + (long)yy * S + x;
+#pragma unroll
+                for (int j = 0; j < 8; j++) {
+                    const int ci = (pl & 1) * 8 + j;
+                    v[u][j] = in && ci < A.C0 ? __ldg(p + (long)ci * A.in_cs) : 0.f;
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < U; u++) {
+                const int e = e0 + u * kTcThreads;
+                if (e < items) *reinterpret_cast<uint4 *>(X + (size_t)e * 16) = pack8(v[u]);
+            }
+        }
+    }
+    __syncthreads();  // the weight images are zero
+    net_weights<2, 4>(A.w1, kNetC, A.C0, W1);
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tm = tmem_base, bars = smem_u32(mbar);
+    const uint32_t bars2 = bars + 8u * (uint32_t)(R + 4), bars3 = bars2 + 8u * (uint32_t)(R + 2);
+    uint32_t last = bars + 8u * (uint32_t)(R + 3);  // completes with the MMAs issued so far
+    bool ok;
+    do {
+        if (tid == 0) net_mma<2, 32, 32>(smem_u32(X), smem_u32(W1), R + 4, tm, bars);
+        net_weights<4, 4>(A.w2, kNetC, kNetC, W2);
+        net_weights<4, 2>(A.w3, A.C3, kNetC, W3);
+        ok = net_hidden(H1, R + 4, y0 - 2, S, A.b1, tm, bars);
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        ok = __syncthreads_and(ok);
+        if (!ok) break;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        last = bars2 + 8u * (uint32_t)(R + 1);
+        if (tid == 0) net_mma<4, 32, 32>(smem_u32(H1), smem_u32(W2), R + 2, tm, bars2);
+        ok = net_hidden(H2, R + 2, y0 - 1, S, A.b2, tm, bars2);
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        ok = __syncthreads_and(ok);
+        if (!ok) break;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        last = bars3 + 8u * (uint32_t)(R - 1);
+        if (tid == 0) net_mma<4, 16, 16>(smem_u32(H2), smem_u32(W3), R, tm, bars3);
+        const int x = (warp & 3) * 32 + (tid & 31);
+        for (int i = warp >> 2; i < R && ok; i += kTcThreads / 128) {
+            ok = __all_sync(0xffffffffu, mbar_wait(bars3 + 8u * (uint32_t)i, 0));
+            if (!ok) break;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            float v[16];
+            tmem_load_row<16>(tm + 16u * (uint32_t)i + ((uint32_t)((warp & 3) * 32) << 16), v);
+            if (x < S && y0 + i < S) {
+                float *o = A.out + base + (long)(y0 + i) * S + x;
+#pragma unroll
+                for (int co = 0; co < 16; co++)
+                    if (co < A.C3) o[(long)co * A.out_cs] = v[co] + __ldg(A.b3 + co);
+            }
+        }
+        ok = __syncthreads_and(ok);
+    } while (0);
+    if (!ok) {
+        // the MMAs did not complete in time: record it and give them one more
+        // bounded wait before the TMEM is freed
+        if (tid == 0 && A.status) atomicCAS(A.status, 0, FEWHA_ERR_TIMEOUT);
+        mbar_wait(last, 0);
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (warp == 0)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tm), "r"(kNetCols) : "memory");
+}
+
 }  // namespace
 
 extern "C" int fewha_conv3x3_fwd_tc(const float *in, long in_bs, long in_cs, int Cin, const float *w,
@@ -326,5 +567,50 @@ extern "C" int fewha_conv3x3_fwd_tc(const float *in, long in_bs, long in_cs, int
     else
         e = launch(k_conv3x3_tc<32>, set32);
     if (e != cudaSuccess) return FEWHA_ERR_CUDA;
+    return cudaGetLastError() == cudaSuccess ? FEWHA_OK : FEWHA_ERR_CUDA;
+}
+
+extern "C" int fewha_convnet_fwd_tc(const float *in, long in_cs, int C0, const float *w1, const float *b1,
+                                    const float *w2, const float *b2, const float *w3, const float *b3, float *out,
+                                    long out_cs, int C3, int ngroups, const int *count, const int *side,
+                                    const long *off, int *status_dev, cudaStream_t s)
+{
+    if (!in || !w1 || !b1 || !w2 || !b2 || !w3 || !b3 || !out || !count || !side || !off || C0 < 1 || C0 > 16 ||
+        C3 < 1 || C3 > 16 || ngroups < 1 || ngroups > kNetGroups)
+        return FEWHA_ERR_ARG;
+    for (int g = 0; g < ngroups; g++)
+        if (count[g] < 1 || count[g] > (1 << 20) || side[g] < 1 || side[g] > kTcM || off[g] < 0) return FEWHA_ERR_ARG;
+    int dev = 0, nsm = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return FEWHA_ERR_CUDA;
+    // Output rows per CTA: least (waves x rows computed over the three layers
+    // plus a fixed part for staging, about ten rows' worth).
+    long best = 0, ctas = 0;
+    int rows = 0;
+    for (int r = kNetRowsMin; r <= kNetRows; r++) {
+        long n = 0;
+        for (int g = 0; g < ngroups; g++) n += (long)count[g] * ((side[g] + r - 1) / r);
+        const long cost = (n + nsm - 1) / nsm * (3 * r + 6 + 10);
+        if (rows == 0 || cost < best) {
+            best = cost;
+            rows = r;
+            ctas = n;
+        }
+    }
+    if (ctas > 0x7FFFFFFFL) return FEWHA_ERR_ARG;
+    NetArgs A{};
+    A.in = in, A.w1 = w1, A.b1 = b1, A.w2 = w2, A.b2 = b2, A.w3 = w3, A.b3 = b3, A.out = out;
+    A.in_cs = in_cs, A.out_cs = out_cs, A.C0 = C0, A.C3 = C3, A.rows = rows, A.ngroups = ngroups, A.status = status_dev;
+    int c0 = 0;
+    for (int g = 0; g < ngroups; g++) {
+        const int tiles = (side[g] + rows - 1) / rows;
+        A.g[g] = NetGroup{side[g], tiles, c0, off[g]};
+        c0 += count[g] * tiles;
+    }
+    if (cudaFuncSetAttribute(k_convnet_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)net_smem(kNetRows)) !=
+        cudaSuccess)
+        return FEWHA_ERR_CUDA;
+    k_convnet_tc<<<(unsigned)ctas, kTcThreads, net_smem(rows), s>>>(A);
     return cudaGetLastError() == cudaSuccess ? FEWHA_OK : FEWHA_ERR_CUDA;
 }

@@ -159,6 +159,8 @@ def load_library(path=LIB_PATH):
     learned = {
         "fewha_conv3x3_fwd": [vp, L, L, I, vp, vp, vp, L, L, I, I, I, I, I, vp],
         "fewha_conv3x3_fwd_tc": [vp, L, L, I, vp, vp, vp, L, L, I, I, I, I, I, vp, vp],
+        "fewha_convnet_fwd_tc": [vp, L, I, vp, vp, vp, vp, vp, vp, vp, L, I, I, C.POINTER(C.c_int),
+                                 C.POINTER(C.c_int), C.POINTER(C.c_long), vp, vp],
         "fewha_conv3x3_bwd_data_relu": [vp, L, L, I, vp, vp, vp, L, L, I, I, I, I, vp],
         "fewha_conv3x3_bwd_data": [vp, L, L, I, vp, vp, L, L, I, I, I, I, vp],
         "fewha_conv3x3_bwd_weight": [vp, L, L, I, vp, L, L, I, I, I, I, vp, vp, I, vp, vp],
@@ -196,7 +198,7 @@ def exported_symbols():
             "fewha_mse_grad", "fewha_adam_step", "fewha_scale", "fewha_learned_targets",
             "fewha_deflate_warm_start", "fewha_mcao_create", "fewha_mcao_n_actuators", "fewha_mcao_fit",
             "fewha_mcao_destroy", "fewha_get_launch_info", "fewha_set_noise", "fewha_read_probe", "fewha_set_pt_bands",
-            "fewha_batch_create_ex", "fewha_batch_tiles", "fewha_conv3x3_fwd_tc", "fewha_store"]
+            "fewha_batch_create_ex", "fewha_batch_tiles", "fewha_conv3x3_fwd_tc", "fewha_convnet_fwd_tc", "fewha_store"]
 
 
 def make_geometry(geom, noise_w, precision="f64", tile=0, grid=0) -> GEOMETRY:

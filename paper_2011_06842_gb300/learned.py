@@ -30,6 +30,7 @@ import numpy as np
 from .fewha import FewhaError, _stream_ptr, load_library
 
 CHANNELS = (4, 32, 32, 5)
+TC_MAX_GROUPS = 8  # most layer sizes of one launch of the whole network
 N_DIR = 5
 
 
@@ -100,6 +101,11 @@ class ConvNet:
                 buf.append(torch.empty((cnt, 32, nl, nl), dtype=torch.float32, device=dev))
             for ci, co in ((c0, c1), (c1, c2), (c2, c3)):
                 ws = max(ws, self.lib.fewha_conv3x3_wgrad_workspace(ci, co, cnt, nl, nl))
+        ng = len(self.groups)
+        self._tc_groups = ((C.c_int * ng)(*[cnt for _, cnt, _ in self.groups]),
+                           (C.c_int * ng)(*[nl for _, _, nl in self.groups]),
+                           (C.c_long * ng)(*[off for off, _, _ in self.groups]))
+        self._hidden = True  # h1, h2 hold the activations of the last forward()
         self.work = torch.empty(max(ws, 1), dtype=torch.float32, device=dev)
         self.loss_part = torch.zeros(512, dtype=torch.float64, device=dev)
 
@@ -115,10 +121,27 @@ class ConvNet:
         """y (5, n) = network(x), x channel k at address x_ptr + 4 * k * x_cs.
         tensor_cores: the convolutions run on the tcgen05 kernel (bfloat16
         operands, FP32 accumulation; inference), else on the FP32 kernel
-        (training: its activations feed the backward pass)."""
+        (training: its activations feed the backward pass).  On the tensor
+        cores the whole network is one launch that keeps the hidden layers on
+        chip; backward() forms them again."""
+        if tensor_cores and len(self.groups) <= TC_MAX_GROUPS:
+            c0, _, _, c3 = CHANNELS
+            p = lambda k: self._p(self.param, k)  # noqa: E731
+            self._ck(self.lib.fewha_convnet_fwd_tc(C.c_void_p(x_ptr), x_cs, c0, p("w1"), p("b1"), p("w2"), p("b2"),
+                                                   p("w3"), p("b3"), C.c_void_p(y.data_ptr()), y.stride(0), c3,
+                                                   len(self.groups), *self._tc_groups, self._tc_status(),
+                                                   _stream_ptr(self.torch)), "convnet")
+            self._hidden = False
+            return y
+        self._hidden = True
         for name, _, launch in self.convolutions(x_ptr, x_cs, y, tensor_cores):
             self._ck(launch(), name)
         return y
+
+    def _tc_status(self):
+        if not hasattr(self, "tc_status"):
+            self.tc_status = self.torch.zeros(1, dtype=self.torch.int32, device=self.param.device)
+        return C.c_void_p(self.tc_status.data_ptr())
 
     def convolutions(self, x_ptr, x_cs, y, tensor_cores=False):
         """The launches of forward(), in order: (name, FLOPs, launch) per 3x3
@@ -127,9 +150,7 @@ class ConvNet:
         lib, s = self.lib, _stream_ptr(self.torch)
         c0, c1, c2, c3 = CHANNELS
         if tensor_cores:
-            if not hasattr(self, "tc_status"):
-                self.tc_status = self.torch.zeros(1, dtype=self.torch.int32, device=self.param.device)
-            st = C.c_void_p(self.tc_status.data_ptr())
+            st = self._tc_status()
             conv = lambda *a: lib.fewha_conv3x3_fwd_tc(*a[:-1], st, a[-1])  # noqa: E731
         else:
             conv = lib.fewha_conv3x3_fwd
@@ -155,6 +176,11 @@ class ConvNet:
         lib, s = self.lib, _stream_ptr(self.torch)
         c0, c1, c2, c3 = CHANNELS
         work = C.c_void_p(self.work.data_ptr())
+        if not self._hidden:
+            for i, (name, _, launch) in enumerate(self.convolutions(x_ptr, x_cs, gy, tensor_cores=True)):
+                if i % 3 < 2:  # the two hidden layers of each group
+                    self._ck(launch(), name)
+            self._hidden = True
         for gi, (off, cnt, nl) in enumerate(self.groups):
             hw = nl * nl
             acc = 1 if gi > 0 else 0

@@ -107,6 +107,58 @@ def test_conv_gradients_at_tile_and_channel_edges(lib, B, Cin, Cout, H, W):
     assert np.abs(gw.cpu().numpy() - rw).max() < 1e-5 * scale and np.abs(gb.cpu().numpy() - rb).max() < 1e-5 * scale
 
 
+@pytest.mark.parametrize("C0,C3,sides", [(4, 5, [(5, 128), (4, 64)]), (1, 1, [(1, 1), (2, 9)]), (16, 16, [(1, 33)]),
+                                         (3, 8, [(40, 127), (1, 2), (7, 16)])])
+def test_whole_network_on_the_tensor_cores(lib, C0, C3, sides):
+    """One launch against the three convolutions one by one on the tensor cores: the same bfloat16 operands and
+    FP32 sums, so equal up to the order of FP32 additions (1e-5 of the output's norm; a hidden value whose last
+    bits differ may round to the neighbouring bfloat16, 2^-8 of one of 288 terms, hence 1e-4)."""
+    _, L = lib
+    rng = np.random.default_rng(C0 + C3)
+    sizes = [cnt * nl * nl for cnt, nl in sides]
+    offs, n = np.concatenate([[0], np.cumsum(sizes)]), sum(sizes) + 3
+    x = dev(rng.standard_normal((C0, n)))
+    ws = [dev(rng.standard_normal(s) * np.sqrt(2.0 / (9 * s[1]))) for s in ((32, C0, 3, 3), (32, 32, 3, 3), (C3, 32, 3, 3))]
+    bs = [dev(0.1 * rng.standard_normal(k)) for k in (32, 32, C3)]
+    out, ref = torch.full((C3, n), 7.0, device="cuda"), torch.full((C3, n), 7.0, device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    ng = len(sides)
+    # channel k at row C0 - 1 - k: a negative channel stride, as over a ring of frames
+    assert L.fewha_convnet_fwd_tc(ptr(x, (C0 - 1) * n), -n, C0, ptr(ws[0]), ptr(bs[0]), ptr(ws[1]), ptr(bs[1]),
+                                  ptr(ws[2]), ptr(bs[2]), ptr(out), n, C3, ng,
+                                  (C.c_int * ng)(*[c for c, _ in sides]), (C.c_int * ng)(*[s for _, s in sides]),
+                                  (C.c_long * ng)(*[int(o) for o in offs[:-1]]), ptr(status), S()) == 0
+    for (cnt, nl), o in zip(sides, offs):
+        hw, o = nl * nl, int(o)
+        h = [torch.empty((cnt, 32, nl, nl), device="cuda") for _ in range(2)]
+        for args in ((ptr(x, (C0 - 1) * n + o), hw, -n, C0, 0, ptr(h[0]), 32 * hw, hw, 32, 1),
+                     (ptr(h[0]), 32 * hw, hw, 32, 1, ptr(h[1]), 32 * hw, hw, 32, 1),
+                     (ptr(h[1]), 32 * hw, hw, 32, 2, ptr(ref, o), hw, n, C3, 0)):
+            xp, xb, xc, ci, k, yp, yb, yc, co, relu = args
+            assert L.fewha_conv3x3_fwd_tc(xp, xb, xc, ci, ptr(ws[k]), ptr(bs[k]), yp, yb, yc, co, cnt, nl, nl, relu,
+                                          ptr(status), S()) == 0
+    assert int(status.item()) == 0
+    assert rel(out.cpu().numpy(), ref.cpu().numpy()) < 1e-4
+    assert torch.all(out[:, -3:] == 7.0)  # nothing written past the images
+
+
+def test_backward_after_the_fused_forward(lib):
+    """Gradients after a tensor-core forward use its hidden layers: equal to those after the three separate
+    tensor-core convolutions."""
+    from paper_2011_06842_gb300.learned import ConvNet
+    net = ConvNet(configs.tiny(), seed=3)
+    g = torch.Generator(device="cuda").manual_seed(1)
+    x, gy = torch.randn(4, net.n, generator=g, device="cuda"), torch.randn(5, net.n, generator=g, device="cuda")
+    y = torch.empty_like(gy)
+    net.forward(x.data_ptr(), net.n, y, tensor_cores=True)
+    net.backward(x.data_ptr(), net.n, gy)
+    fused = net.grad.clone()
+    for name, _, launch in net.convolutions(x.data_ptr(), net.n, y, tensor_cores=True):
+        assert launch() == 0, name
+    net.backward(x.data_ptr(), net.n, gy)
+    assert torch.equal(fused, net.grad)
+
+
 def test_conv_strided_channels(lib):
     """Channels as whole vectors (stride n, and -n over a ring, newest first)."""
     _, L = lib
