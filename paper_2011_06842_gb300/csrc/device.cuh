@@ -283,16 +283,51 @@ __device__ __forceinline__ A warp_sum_t(A v)
     return v;
 }
 
+// Warp sums of NV <= 32 FP64 values: lane L returns the sum of value
+// bitreverse5(L) (if below NV).  At each level a lane hands one of every two
+// values to its partner and adds the partner's half of the other, so the
+// warp issues NV/2 + NV/4 + ... additions instead of 5 NV (the FP64 pipe takes a
+// warp instruction every 64 cycles: for 18 values of 16 warps 2.7 us instead
+// of 12).
+template <int NV>
+__device__ __forceinline__ double warp_sum_transposed(const double (&v)[NV])
+{
+    const int lane = threadIdx.x & 31;
+    double w[NV];
+#pragma unroll
+    for (int i = 0; i < NV; i++) w[i] = v[i];
+    int n = NV;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const bool hi = lane & o;
+#pragma unroll
+        for (int j = 0; j < NV / 2; j++)
+            if (2 * j + 1 < n) {
+                const double keep = hi ? w[2 * j + 1] : w[2 * j], give = hi ? w[2 * j] : w[2 * j + 1];
+                w[j] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+            }
+        if (n & 1) w[n / 2] = w[n - 1] + __shfl_xor_sync(0xffffffffu, w[n - 1], o);
+        n = (n + 1) / 2;
+    }
+    return w[0];
+}
+
 // Block-wide sum of NV values per thread, written as partials of this CTA.
 template <int NV, typename A>
 __device__ void block_partials(A (&v)[NV], double *part, const int (&slot)[NV], double *sred, int cta)
 // sred: shared scratch of NV * 32 doubles; cta: this CTA's rank in its group
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    if constexpr (sizeof(A) == 8 && NV > 1 && NV <= 32) {
+        const int i = __brev(lane) >> 27;
+        const double s = warp_sum_transposed<NV>(v);
+        if (i < NV) sred[i * 32 + warp] = s;
+    } else {
 #pragma unroll
-    for (int i = 0; i < NV; i++) {
-        A s = warp_sum_t(v[i]);
-        if (lane == 0) sred[i * 32 + warp] = (double)s;
+        for (int i = 0; i < NV; i++) {
+            A s = warp_sum_t(v[i]);
+            if (lane == 0) sred[i * 32 + warp] = (double)s;
+        }
     }
     __syncthreads();
     if constexpr (NV <= kThreads / 32) {
@@ -590,10 +625,14 @@ __device__ __forceinline__ Taps<T, L> load_taps(const Geo<T> &G)
 
 // One run of `run` output pairs starting at pair m0 of the line at base
 // (element stride es), into out[0 .. 2 kRun).
-template <typename T, int L, bool SYNTH>
-__device__ __forceinline__ void dwt_run(const T *base, int es, int N, int half, int run, int m0,
+// RUN > 0: `run` is that constant, and only its pairs are computed.  FP64 sums
+// are FMA chains: two FP64 instructions per tap pair instead of three.
+template <typename T, int L, bool SYNTH, int RUN = 0>
+__device__ __forceinline__ void dwt_run(const T *base, int es, int N, int half, int run_, int m0,
                                         const Taps<T, L> &tp, T (&out)[2 * kRun])
 {
+    const int run = RUN > 0 ? RUN : run_;
+    constexpr int NQ = RUN > 0 ? RUN : kRun;
     constexpr int Lh = L / 2;
     if (SYNTH) {
         T wa[kRun + Lh - 1], wd[kRun + Lh - 1];  // a_{m0-Lh+1 .. m0+kRun-1}, same for d
@@ -608,13 +647,18 @@ __device__ __forceinline__ void dwt_run(const T *base, int es, int N, int half, 
             }
         }
 #pragma unroll
-        for (int q = 0; q < kRun; q++) {
+        for (int q = 0; q < NQ; q++) {
             T x0 = 0, x1 = 0;
 #pragma unroll
             for (int u = 0; u < Lh; u++) {
                 const T a = wa[q + Lh - 1 - u], d = wd[q + Lh - 1 - u];
-                x0 += tp.h[2 * u] * a + tp.g[2 * u] * d;
-                x1 += tp.h[2 * u + 1] * a + tp.g[2 * u + 1] * d;
+                if constexpr (sizeof(T) == 8) {
+                    x0 = fma(tp.g[2 * u], d, fma(tp.h[2 * u], a, x0));
+                    x1 = fma(tp.g[2 * u + 1], d, fma(tp.h[2 * u + 1], a, x1));
+                } else {
+                    x0 += tp.h[2 * u] * a + tp.g[2 * u] * d;
+                    x1 += tp.h[2 * u + 1] * a + tp.g[2 * u + 1] * d;
+                }
             }
             out[2 * q] = x0;
             out[2 * q + 1] = x1;
@@ -625,7 +669,7 @@ __device__ __forceinline__ void dwt_run(const T *base, int es, int N, int half, 
         for (int i = 0; i < 2 * kRun + L - 2; i++)
             wx[i] = (i < 2 * run + L - 2) ? base[((2 * m0 + i) & (N - 1)) * es] : T(0);
 #pragma unroll
-        for (int q = 0; q < kRun; q++) {
+        for (int q = 0; q < NQ; q++) {
             T a = 0, d = 0;
 #pragma unroll
             for (int u = 0; u < L; u++) {
@@ -649,6 +693,27 @@ __device__ __forceinline__ void dwt_store(T *base, int es, int half, int run, in
             base[p0 * es] = out[2 * q];
             base[p1 * es] = out[2 * q + 1];
         }
+    }
+}
+
+// The lines of one in-place pass in runs of RUN pairs: a line's outputs
+// overwrite only that line, so the lanes of one warp read the whole line into
+// registers, synchronise and write it back; a warp takes 32 / (runs per line)
+// lines at once.  N <= FEWHA_MAX_GRID = 128: at most 16 runs of 4 pairs per line;
+// runs of 2 and 1 are used below 64 x 64 and 32 x 32: at most 16 per line too.
+template <typename T, int L, bool SYNTH, int RUN>
+__device__ __forceinline__ void dwt_lines(const T *src, T *dst, int es, int ls, int N, int half, const Taps<T, L> &tp)
+{
+    const int nr = half / RUN, lpw = 32 / nr;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int sub = lane / nr, m0 = (lane - sub * nr) * RUN;
+    for (int line0 = warp * lpw; line0 < N; line0 += nw * lpw) {
+        const int line = line0 + sub;
+        const bool act = line < N && sub < lpw;
+        T out[2 * kRun];
+        if (act) dwt_run<T, L, SYNTH, RUN>(src + line * ls, es, N, half, RUN, m0, tp, out);
+        __syncwarp();
+        if (act) dwt_store<SYNTH>(dst + line * ls, es, half, RUN, m0, out);
     }
 }
 
@@ -676,21 +741,17 @@ __device__ void dwt_pass(const T *src, T *dst, int P, int lgN, const Geo<T> &G)
         }
         __syncthreads();
     } else {
-        // in place (FP64): a line's outputs overwrite only that line, so the
-        // lanes of one warp read the whole line into registers, synchronise
-        // and write it back; a warp takes 32 / (runs per line) lines at once
-        // (N <= FEWHA_MAX_GRID = 128: at most 16 runs of 4 pairs per line)
-        const int nr = half / run, lpw = 32 / nr;
-        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-        const int sub = lane / nr, m0 = (lane - sub * nr) * run;
-        for (int line0 = warp * lpw; line0 < N; line0 += nw * lpw) {
-            const int line = line0 + sub;
-            const bool act = line < N;
-            T out[2 * kRun];
-            if (act) dwt_run<T, L, SYNTH>(src + line * ls, es, N, half, run, m0, tp, out);
-            __syncwarp();
-            if (act) dwt_store<SYNTH>(dst + line * ls, es, half, run, m0, out);
-        }
+        // in place (FP64).  The pass is bound by the FP64 pipes, one per quarter
+        // of the SM: pairs per run as few as it takes to give every quarter two
+        // warps (a level of 8 x 8 has two pairs for each of 16 threads or one
+        // for each of 32; with four per thread one warp computed a 16 x 16
+        // level alone, 1.6 us instead of 0.4).
+        if (half >= kRun && (N * half) / kRun >= 8 * 32)
+            dwt_lines<T, L, SYNTH, kRun>(src, dst, es, ls, N, half, tp);
+        else if (half >= 2 && (N * half) / 2 >= 8 * 32)
+            dwt_lines<T, L, SYNTH, 2>(src, dst, es, ls, N, half, tp);
+        else
+            dwt_lines<T, L, SYNTH, 1>(src, dst, es, ls, N, half, tp);
         __syncthreads();
     }
 }

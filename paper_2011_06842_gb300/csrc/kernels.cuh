@@ -1183,12 +1183,18 @@ struct Impl : ImplBase {
         }
     };
 
-    // Form of the chain for `group` CTAs per vector.  FP64: split whenever a
-    // group can be (a layer's CTA is bound by its FP64 units).  FP32: from four
-    // CTAs per layer; below, the two tiled kernels' launches and rounds cost
-    // what they take off the layers' CTAs (9 ELT layers, 5 vectors, 30 CTAs
-    // each: 94.7 us split, 91.9 us whole).
-    bool op_split(int group) const { return group >= (sizeof(T) == 8 ? 2 : 4) * P.L; }
+    // Form of the chain for `group` CTAs per vector.  Split costs two more
+    // kernels (four with two tiled levels): it pays where the finest level keeps
+    // a layer's CTA longer than that.  FP64: layers from 64^2 (12 FMAs per node
+    // at two per clock, 13 us).  FP32: layers of 128^2 and four CTAs per layer;
+    // with fewer, the tiled kernels take several rounds (9 ELT layers, 5 vectors
+    // of 30 CTAs: 94.7 us split, 91.9 us whole).
+    bool op_split(int group) const
+    {
+        int nmax = 0;
+        for (int l = 0; l < P.L; l++) nmax = std::max(nmax, P.geom.layers[l].n);
+        return sizeof(T) == 8 ? nmax >= 64 && group >= 2 * P.L : nmax >= 128 && group >= 4 * P.L;
+    }
 
     // nodal = W^{-1} x; group: CTAs per vector
     template <class A>

@@ -233,7 +233,8 @@ __device__ __forceinline__ void phase_init(const Args<T, S> &A, const Basis &b, 
 #pragma unroll
         for (int j = 0; j < kK; j++) qj[j] = j < kv ? __ldg(sq[j] + e) : T(0);
 #pragma unroll
-        for (int j = 0; j < kK; j++) acc[j] += (Acc)qj[j] * (Acc)z;
+        for (int j = 0; j < kK; j++)
+            if (sizeof(T) == 4 || j < kv) acc[j] += (Acc)qj[j] * (Acc)z;  // no FP64 work for absent directions
     }
     int slots[kK + 2];
     for (int j = 0; j < kK; j++) slots[j] = kSlotInit + j;
