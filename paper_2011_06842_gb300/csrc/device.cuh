@@ -79,6 +79,7 @@ struct Geo {
     int lay_n[FEWHA_MAX_LAYERS], lay_J[FEWHA_MAX_LAYERS];
     long lay_off[FEWHA_MAX_LAYERS + 1];
     long ll_off[FEWHA_MAX_LAYERS + 1];  // (n_l/2)^2 blocks: level-1 approximation scratch
+    int split_min;              // CTAs of a group from which the split form is used (split_levels)
     int depth;                  // split form: finest wavelet levels tiled over all CTAs (split_depth)
     T inv_delta[FEWHA_MAX_LAYERS];
     int n_taps;
@@ -625,6 +626,13 @@ __device__ __forceinline__ Taps<T, L> load_taps(const Geo<T> &G)
 
 // One run of `run` output pairs starting at pair m0 of the line at base
 // (element stride es), into out[0 .. 2 kRun).
+// One tap pair of a synthesis sum.  FP64: two FMAs instead of a product, an FMA
+// and an addition.
+template <typename T>
+__device__ __forceinline__ void synth_acc(T &x, T h, T a, T g, T d)
+{
+    x = fma(g, d, fma(h, a, x));
+}
 // RUN > 0: `run` is that constant, and only its pairs are computed.  FP64 sums
 // are FMA chains: two FP64 instructions per tap pair instead of three.
 template <typename T, int L, bool SYNTH, int RUN = 0>
@@ -653,8 +661,8 @@ __device__ __forceinline__ void dwt_run(const T *base, int es, int N, int half, 
             for (int u = 0; u < Lh; u++) {
                 const T a = wa[q + Lh - 1 - u], d = wd[q + Lh - 1 - u];
                 if constexpr (sizeof(T) == 8) {
-                    x0 = fma(tp.g[2 * u], d, fma(tp.h[2 * u], a, x0));
-                    x1 = fma(tp.g[2 * u + 1], d, fma(tp.h[2 * u + 1], a, x1));
+                    synth_acc(x0, tp.h[2 * u], a, tp.g[2 * u], d);
+                    synth_acc(x1, tp.h[2 * u + 1], a, tp.g[2 * u + 1], d);
                 } else {
                     x0 += tp.h[2 * u] * a + tp.g[2 * u] * d;
                     x1 += tp.h[2 * u + 1] * a + tp.g[2 * u + 1] * d;

@@ -912,6 +912,16 @@ struct Impl : ImplBase {
             const long h = P.geom.layers[l].n / 2;
             G.ll_off[l + 1] = G.ll_off[l] + h * h;
         }
+        // The split form costs an iteration two phases and two barriers, 4.4 us
+        // each in FP32 and 7 to 10 us in FP64 on 152 CTAs; the finest level on
+        // the layer's own CTA costs about 2 us at 64^2 in FP32 and 3 us at 32^2
+        // in FP64 (twice FP32's next size, and four times FP64's, is more than
+        // the phase).
+        {
+            int nmax = 0;
+            for (int l = 0; l < P.L; l++) nmax = std::max(nmax, P.geom.layers[l].n);
+            G.split_min = nmax > (sizeof(T) == 8 ? 32 : 64) ? 2 * P.L : kMaxCtas + 1;
+        }
         // two tiled levels where a layer CTA's block would be 64^2 in FP64 (split_depth)
         {
             int nmax = 0;
@@ -1090,7 +1100,7 @@ struct Impl : ImplBase {
         out->ctas = ncta;
         out->threads = kThreads;
         out->smem_bytes = (long)smem;
-        out->split_levels = ncta >= 2 * P.L ? 1 : 0;
+        out->split_levels = ncta >= base.geo.split_min ? 1 : 0;
         out->staged_tables = base.geo.stage_tab;
         out->wfs_tile_y = base.geo.tile_y;
         out->wfs_tile_x = base.geo.tile_x;
@@ -1184,16 +1194,13 @@ struct Impl : ImplBase {
     };
 
     // Form of the chain for `group` CTAs per vector.  Split costs two more
-    // kernels (four with two tiled levels): it pays where the finest level keeps
-    // a layer's CTA longer than that.  FP64: layers from 64^2 (12 FMAs per node
-    // at two per clock, 13 us).  FP32: layers of 128^2 and four CTAs per layer;
-    // with fewer, the tiled kernels take several rounds (9 ELT layers, 5 vectors
-    // of 30 CTAs: 94.7 us split, 91.9 us whole).
+    // kernels (four with two tiled levels) and pays where the solver's split form
+    // does (Geo::split_min); in FP32 from four CTAs per layer: with fewer, the
+    // tiled kernels take several rounds (9 ELT layers, 5 vectors of 30 CTAs:
+    // 94.7 us split, 91.9 us whole).
     bool op_split(int group) const
     {
-        int nmax = 0;
-        for (int l = 0; l < P.L; l++) nmax = std::max(nmax, P.geom.layers[l].n);
-        return sizeof(T) == 8 ? nmax >= 64 && group >= 2 * P.L : nmax >= 128 && group >= 4 * P.L;
+        return group >= base.geo.split_min && (sizeof(T) == 8 || group >= 4 * P.L);
     }
 
     // nodal = W^{-1} x; group: CTAs per vector
@@ -1638,7 +1645,7 @@ struct Impl : ImplBase {
                 CK(cudaLaunchKernelEx(&cfg, k_solve_persistent<T, S, false>, A));
             return launch_check();
         }
-        const bool deep = A.geo.depth > 1 && ncta >= 2 * P.L;  // split_levels, split_depth
+        const bool deep = A.geo.depth > 1 && ncta >= A.geo.split_min;  // split_levels, split_depth
         k_rhs_wfs<T, S><<<ncta, kThreads, smem, s>>>(A);
         k_rhs_gather<T, S><<<ncta, kThreads, smem, s>>>(A);
         k_rhs_D1<T, S, 0><<<ncta, kThreads, smem, s>>>(A);

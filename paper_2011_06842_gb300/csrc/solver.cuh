@@ -286,18 +286,20 @@ __device__ __forceinline__ void for_detail_vectors(const Geo<T> &G, long lo, lon
 }
 
 // Two ways to run the layers' transforms, chosen per instance:
-//   split (at least twice as many CTAs as layers): the finest level is tiled
+//   split (at least twice as many CTAs as layers, and layers large enough,
+//     Geo::split_min): the finest level is tiled
 //     over all CTAs (A2, D1); the first L CTAs own one layer's (n/2)^2 block
 //     each, run its coarser levels in shared memory and take no detail
 //     coefficients (the block transforms are then the critical path);
-//   whole (fewer CTAs, e.g. the small instances of a batch): each layer's CTA
+//   whole (fewer CTAs, e.g. the small instances of a batch, or smaller layers):
+//     each layer's CTA
 //     updates the whole layer, runs every level in shared memory and updates
 //     the layer again after the forward transform; A2 and D1 are empty, so an
 //     iteration has four grid barriers instead of six.
 template <typename T, typename S>
 __device__ __forceinline__ bool split_levels(const Args<T, S> &A)
 {
-    return A.ncta >= 2 * A.geo.L;
+    return A.ncta >= A.geo.split_min;
 }
 
 // body(global element, index in the layer CTA's block), one W-vector per call
@@ -734,8 +736,8 @@ __device__ void fine_synthesis(const Args<T, S> &A, const T *pk, T *sm)
                 for (int u = 0; u < Lh; u++) {
                     const int r = i + Lh - 1 - u;
                     const T a = lo[r * WC], d = hi[r * WC];
-                    x0 = fma(tp.g[2 * u], d, fma(tp.h[2 * u], a, x0));
-                    x1 = fma(tp.g[2 * u + 1], d, fma(tp.h[2 * u + 1], a, x1));
+                    synth_acc(x0, tp.h[2 * u], a, tp.g[2 * u], d);
+                    synth_acc(x1, tp.h[2 * u + 1], a, tp.g[2 * u + 1], d);
                 }
                 mid[2 * i * (2 * WC) + cc] = x0;
                 mid[(2 * i + 1) * (2 * WC) + cc] = x1;
@@ -749,8 +751,8 @@ __device__ void fine_synthesis(const Args<T, S> &A, const T *pk, T *sm)
                 for (int u = 0; u < Lh; u++) {
                     const int c = j + Lh - 1 - u;
                     const T a = row[c], d = row[WC + c];
-                    x0 = fma(tp.g[2 * u], d, fma(tp.h[2 * u], a, x0));
-                    x1 = fma(tp.g[2 * u + 1], d, fma(tp.h[2 * u + 1], a, x1));
+                    synth_acc(x0, tp.h[2 * u], a, tp.g[2 * u], d);
+                    synth_acc(x1, tp.h[2 * u + 1], a, tp.g[2 * u + 1], d);
                 }
                 const long o = (long)(2 * p0y + yy) * N + 2 * (p0x + j);
                 if constexpr (LV == 0) {
