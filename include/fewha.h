@@ -391,6 +391,27 @@ int fewha_conv3x3_fwd(const float *in, long in_bs, long in_cs, int Cin, const fl
 int fewha_conv3x3_fwd_tc(const float *in, long in_bs, long in_cs, int Cin, const float *w, const float *bias,
                          float *out, long out_bs, long out_cs, int Cout, int B, int H, int W, int relu,
                          int *status_dev, cudaStream_t s);
+/* The network conv(C0 -> C) ReLU conv(C -> C) ReLU conv(C -> C3) in FP32 over
+ * groups of equal-size images (the layers of each size), each convolution and
+ * each gradient one launch for all groups.  Image i of group g starts off[g] +
+ * i side[g]^2 floats into a channel of x, y and gy (channel strides x_cs, y_cs,
+ * gy_cs); h1, h2 (hidden activations) and g1, g2 (their gradients) are arrays of
+ * count[g] x C x side[g] x side[g].  fewha_convnet_fwd writes h1, h2 and y;
+ * fewha_convnet_bwd reads them and writes g1, g2 and the parameter gradients gw,
+ * gb of sum gy y; workspace: at least min(152, sum over groups of count
+ * ceil(side / 16)^2) (C max(C, C0, C3) 9 + max(C, C3)) floats. */
+#define FEWHA_NET_GROUPS 8
+typedef struct fewha_net {
+    int C0, C, C3, ngroups;
+    int count[FEWHA_NET_GROUPS], side[FEWHA_NET_GROUPS];
+    long off[FEWHA_NET_GROUPS];
+    float *h1[FEWHA_NET_GROUPS], *h2[FEWHA_NET_GROUPS], *g1[FEWHA_NET_GROUPS], *g2[FEWHA_NET_GROUPS];
+    const float *w[3], *b[3];
+    float *gw[3], *gb[3];
+} fewha_net;
+int fewha_convnet_fwd(const fewha_net *net, const float *x, long x_cs, float *y, long y_cs, cudaStream_t s);
+int fewha_convnet_bwd(const fewha_net *net, const float *x, long x_cs, const float *gy, long gy_cs, float *workspace,
+                      cudaStream_t s);
 /* fewha_convnet_fwd_tc: the network conv(C0 -> 32) ReLU conv(32 -> 32) ReLU
  *   conv(32 -> C3) in one launch, with the arithmetic of three
  *   fewha_conv3x3_fwd_tc calls; C0, C3 <= 16.  Image i of group g (count[g]

@@ -29,8 +29,9 @@ constexpr int TX = 32;    // output tile width (4 pixels per thread)
 constexpr int TY = 16;    // output tile height
 constexpr int PX = 4;     // adjacent pixels per thread
 constexpr int CO_T = 8;   // output channels per block
-constexpr int CI_T = 8;   // input channels staged per step
+constexpr int CI_T = 4;   // input channels staged per step
 constexpr int NT = TX * TY / PX;
+constexpr int CONV_CTAS = 6;  // CTAs per SM (registers and shared memory allow them)
 constexpr int TP = TX + 4;  // pitch of a staged row: x0-1 .. x0+TX plus slack, 16-byte rows
 
 // out[b][co][y][x] = act(bias[co] + sum_ci sum_{ky,kx} w[co][ci][ky][kx] in[b][ci][y+ky-1][x+kx-1])
@@ -47,24 +48,52 @@ constexpr int TP = TX + 4;  // pitch of a staged row: x0-1 .. x0+TX plus slack, 
 // FMAs per thread, against 60 for 288 with two vertically adjacent pixels and
 // single loads.  Input tiles and weights of the next CI_T channels are copied
 // asynchronously while the present ones are used.
-__global__ void __launch_bounds__(NT) k_conv3x3(const float *__restrict__ in, long in_bs, long in_cs, int Cin,
-                                                const float *__restrict__ w, const float *__restrict__ bias,
-                                                float *__restrict__ out, long out_bs, long out_cs, int Cout, int H,
-                                                int W, int relu, int wt_mode, const float *__restrict__ mask)
+//
+// A launch covers up to kMaxGroups groups of equal-size images (the layers of
+// each size): a group of small images alone leaves most SMs idle.
+constexpr int kMaxGroups = 8;
+
+struct ConvGroup {
+    const float *in, *mask;
+    float *out;
+    long in_bs, in_cs, out_bs, out_cs;
+    int H, W, tiles_x, tiles, blk0;  // tiles per image, first block
+};
+struct ConvArgs {
+    ConvGroup g[kMaxGroups];
+    const float *w, *bias;
+    int ng, Cin, Cout, relu, wt_mode;
+};
+
+__global__ void __launch_bounds__(NT, CONV_CTAS) k_conv3x3(const __grid_constant__ ConvArgs A)
 {
     __shared__ __align__(16) float tile[2][CI_T][TY + 2][TP];
     __shared__ __align__(16) float wsh[2][CI_T][9][CO_T];
+    int gi = 0;
+    while (gi + 1 < A.ng && (int)blockIdx.x >= A.g[gi + 1].blk0) gi++;
+    const ConvGroup &G = A.g[gi];
+    const float *__restrict__ w = A.w, *__restrict__ bias = A.bias, *__restrict__ mask = G.mask;
+    float *__restrict__ out = G.out;
+    const long in_cs = G.in_cs, out_bs = G.out_bs, out_cs = G.out_cs;
+    const int Cin = A.Cin, Cout = A.Cout, H = G.H, W = G.W, relu = A.relu, wt_mode = A.wt_mode;
     const int tx = (threadIdx.x % (TX / PX)) * PX, ty = threadIdx.x / (TX / PX);
-    const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
-    const int nco = (Cout + CO_T - 1) / CO_T;
-    const int b = blockIdx.z / nco, co0 = (blockIdx.z % nco) * CO_T;
-    const float *inb = in + (long)b * in_bs;
+    const int nco = (Cout + CO_T - 1) / CO_T, blk = (int)blockIdx.x - G.blk0;
+    const int t = blk % G.tiles, z = blk / G.tiles;
+    const int x0 = (t % G.tiles_x) * TX, y0 = (t / G.tiles_x) * TY;
+    const int b = z / nco, co0 = (z % nco) * CO_T;
+    const float *__restrict__ inb = G.in + (long)b * G.in_bs;
     auto stage = [&](int s, int ci0) {
-        for (int e = threadIdx.x; e < CI_T * (TY + 2) * (TX + 2); e += NT) {
-            const int c = e / ((TY + 2) * (TX + 2)), r = (e / (TX + 2)) % (TY + 2), q = e % (TX + 2);
-            const int y = y0 + r - 1, x = x0 + q - 1;
-            const bool ok = ci0 + c < Cin && y >= 0 && y < H && x >= 0 && x < W;
-            cp4(&tile[s][c][r][q], ok ? inb + (long)(ci0 + c) * in_cs + (long)y * W + x : inb, ok);
+        // a warp per row of 34 pixels: lanes 0..31, then two lanes for the rest
+        static_assert(TX == 32, "a row is a warp and two pixels");
+        const int lane = threadIdx.x & 31, x = x0 - 1 + lane;
+        const bool okx = x >= 0 && x < W, okt = lane < 2 && x + 32 < W;
+        for (int rr = threadIdx.x >> 5; rr < CI_T * (TY + 2); rr += NT / 32) {
+            const int c = rr / (TY + 2), r = rr - c * (TY + 2), y = y0 + r - 1;
+            const bool row = ci0 + c < Cin && y >= 0 && y < H;
+            const float *src = inb + (long)(ci0 + c) * in_cs + (long)y * W + x;
+            float *dst = &tile[s][c][r][lane];
+            cp4(dst, row && okx ? src : inb, row && okx);
+            if (lane < 2) cp4(dst + 32, row && okt ? src + 32 : inb, row && okt);
         }
         for (int e = threadIdx.x; e < CO_T * CI_T * 9; e += NT) {
             const int k = e % 9, j = wt_mode ? (e / 9) % CO_T : e / (9 * CI_T);
@@ -132,43 +161,51 @@ __global__ void __launch_bounds__(NT) k_conv3x3(const float *__restrict__ in, lo
     }
 }
 
-// Partial weight/bias gradients.  A CTA takes spatial tiles of TS x TS pixels
+// Partial weight/bias gradients.  A CTA takes spatial tiles of TS x TH pixels
 // (tile blockIdx.x, + gridDim.x, ...) and one block of 4 CG output times 2 IG
-// input channels; the tile's gradients and inputs are staged in shared memory
+// input channels; the next tile's gradients and inputs are copied to shared
+// memory while the present one is used,
 // and a thread keeps 4 x 2 x 9 sums in registers for its slice of the tile's
-// rows (256 / (CG IG) slices), so four pixels cost it 4 + 12 shared loads for
+// pixels (512 / (CG IG) slices), so four pixels cost it 4 + 12 shared loads for
 // 288 FMAs (one output value per thread read two operands from shared memory
 // for every FMA).  The slices are summed in slice order at the end.  With the
 // parallel sum of the partials below and the four-pixel convolution above, a
 // training step on the ELT layers (5 x 128^2 and 4 x 64^2) went from 1171 to
 // 596 us.
-constexpr int TS = 16;           // spatial tile of the weight gradient
-constexpr int WG_T = 256;        // threads
-constexpr int WG_CTAS = 304;     // CTAs of one launch: two per SM, so that one stages while the other computes
-constexpr int GP = TS * TS + 4;  // channel pitch of the staged gradients: 8 channels on 8 different 16-byte banks
+constexpr int TS = 16;           // width of the spatial tile; the workspace counts TS x TS tiles
+constexpr int TH = 8;            // its height: 16 x 8 tiles spread over the CTAs more evenly than 16 x 16
+constexpr int WG_T = 512;        // threads
+constexpr int WG_CTAS = 152;     // CTAs of one launch, one per SM: the fewer, the fewer partials to add in FP64
+constexpr int GP = TH * TS + 4;  // channel pitch of the staged gradients: 8 channels on 8 different 16-byte banks
 constexpr int IW = TS + 4;       // row pitch of the staged inputs
-constexpr int IP = (TS + 2) * IW + 4;  // channel pitch of the staged inputs (odd multiple of 16 bytes)
+constexpr int IP = (TH + 2) * IW + 4;  // channel pitch of the staged inputs (odd multiple of 16 bytes)
+
+struct WgradGroup {
+    const float *in, *gout;
+    long in_bs, in_cs, gout_bs, gout_cs;
+    int H, W, tiles_x, tiles, t0;  // tiles per image, first tile
+};
+struct WgradArgs {
+    WgradGroup g[kMaxGroups];
+    float *part;
+    int ng, Cin, Cout, ntiles;
+};
 
 template <int CG, int IG>
 constexpr size_t wg_smem()
 {
-    const size_t tiles = (size_t)(4 * CG * GP + 2 * IG * IP), sums = (size_t)WG_T * 72;
+    const size_t tiles = 2 * (size_t)(4 * CG * GP + 2 * IG * IP), sums = (size_t)WG_T * 72;
     return (tiles > sums ? tiles : sums) * sizeof(float);
 }
 
 template <int CG, int IG>
-__global__ void __launch_bounds__(WG_T, 2)
-    k_conv3x3_wgrad_partial(const float *__restrict__ in, long in_bs, long in_cs, int Cin,
-                            const float *__restrict__ gout, long gout_bs, long gout_cs, int Cout, int H, int W,
-                            int ntiles, float *__restrict__ part)
+__global__ void __launch_bounds__(WG_T, 1) k_conv3x3_wgrad_partial(const __grid_constant__ WgradArgs A)
 {
     extern __shared__ __align__(16) float wg_sm[];
-    constexpr int COB = 4 * CG, CIB = 2 * IG, NS = WG_T / (CG * IG), RS = TS / NS;
-    static_assert(NS * CG * IG == WG_T && NS * RS == TS, "slices cover the tile");
-    float *tg = wg_sm, *tin = wg_sm + COB * GP;
-    const int co0 = blockIdx.y * COB, ci0 = blockIdx.z * CIB;
+    constexpr int COB = 4 * CG, CIB = 2 * IG, NS = WG_T / (CG * IG), BUF = COB * GP + CIB * IP;
+    static_assert(NS * CG * IG == WG_T && (TH * TS / 4) % NS == 0, "slices cover the tile");
+    const int co0 = blockIdx.y * COB, ci0 = blockIdx.z * CIB, Cin = A.Cin, Cout = A.Cout;
     const int cg = threadIdx.x % CG, ig = (threadIdx.x / CG) % IG, slice = threadIdx.x / (CG * IG);
-    const int tiles_x = (W + TS - 1) / TS, tiles_y = (H + TS - 1) / TS;
     float acc[4][2][9];
 #pragma unroll
     for (int j = 0; j < 4; j++)
@@ -176,58 +213,71 @@ __global__ void __launch_bounds__(WG_T, 2)
         for (int i = 0; i < 2; i++)
 #pragma unroll
             for (int k = 0; k < 9; k++) acc[j][i][k] = 0.f;
-    constexpr int BT = WG_T / COB;  // threads per bias channel
+    constexpr int BT = WG_T / COB < 32 ? WG_T / COB : 32;  // threads per bias channel
     float bsum = 0.f;
-    for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
-        const int b = t / (tiles_x * tiles_y), tile = t - b * (tiles_x * tiles_y);
-        const int x0 = (tile % tiles_x) * TS, y0 = (tile / tiles_x) * TS;
-        const float *gb = gout + (long)b * gout_bs, *ib = in + (long)b * in_bs;
-        for (int e = threadIdx.x; e < COB * TS * TS; e += WG_T) {
-            const int c = e / (TS * TS), r = (e / TS) % TS, q = e % TS, y = y0 + r, x = x0 + q;
+    // asynchronous copy of tile t into buffer s
+    auto stage = [&](int s, int t) {
+        int gi = 0;
+        while (gi + 1 < A.ng && t >= A.g[gi + 1].t0) gi++;
+        const WgradGroup &G = A.g[gi];
+        const int H = G.H, W = G.W, lt = t - G.t0, b = lt / G.tiles, tile = lt - b * G.tiles;
+        const int x0 = (tile % G.tiles_x) * TS, y0 = (tile / G.tiles_x) * TH;
+        const float *gb = G.gout + (long)b * G.gout_bs, *ib = G.in + (long)b * G.in_bs;
+        float *tg = wg_sm + s * BUF, *tin = tg + COB * GP;
+        for (int e = threadIdx.x; e < COB * TH * TS; e += WG_T) {
+            const int c = e / (TH * TS), r = (e / TS) % TH, q = e % TS, y = y0 + r, x = x0 + q;
             const bool ok = co0 + c < Cout && y < H && x < W;
-            cp4(tg + c * GP + r * TS + q, ok ? gb + (long)(co0 + c) * gout_cs + (long)y * W + x : gout, ok);
+            cp4(tg + c * GP + r * TS + q, ok ? gb + (long)(co0 + c) * G.gout_cs + (long)y * W + x : gb, ok);
         }
-        for (int e = threadIdx.x; e < CIB * (TS + 2) * (TS + 2); e += WG_T) {
-            const int c = e / ((TS + 2) * (TS + 2)), r = (e / (TS + 2)) % (TS + 2), q = e % (TS + 2);
+        for (int e = threadIdx.x; e < CIB * (TH + 2) * (TS + 2); e += WG_T) {
+            const int c = e / ((TH + 2) * (TS + 2)), r = (e / (TS + 2)) % (TH + 2), q = e % (TS + 2);
             const int y = y0 + r - 1, x = x0 + q - 1;
             const bool ok = ci0 + c < Cin && y >= 0 && y < H && x >= 0 && x < W;
-            cp4(tin + c * IP + r * IW + q, ok ? ib + (long)(ci0 + c) * in_cs + (long)y * W + x : in, ok);
+            cp4(tin + c * IP + r * IW + q, ok ? ib + (long)(ci0 + c) * G.in_cs + (long)y * W + x : ib, ok);
         }
         cp_commit();
-        cp_wait<0>();
-        __syncthreads();
-        for (int r = slice * RS; r < slice * RS + RS; r++) {
-#pragma unroll 1
-            for (int x = 0; x < TS; x += 4) {
-                float4 g[4];
-#pragma unroll
-                for (int j = 0; j < 4; j++)
-                    g[j] = *reinterpret_cast<const float4 *>(tg + (cg + CG * j) * GP + r * TS + x);
-#pragma unroll
-                for (int i = 0; i < 2; i++)
-#pragma unroll
-                    for (int ky = 0; ky < 3; ky++) {
-                        const float *row = tin + (ig + IG * i) * IP + (r + ky) * IW + x;
-                        const float4 va = *reinterpret_cast<const float4 *>(row);
-                        const float2 vb = *reinterpret_cast<const float2 *>(row + 4);
-                        const float v[6] = {va.x, va.y, va.z, va.w, vb.x, vb.y};
-#pragma unroll
-                        for (int kx = 0; kx < 3; kx++)
-#pragma unroll
-                            for (int j = 0; j < 4; j++) {
-                                float a = acc[j][i][3 * ky + kx];
-                                a += g[j].x * v[kx];
-                                a += g[j].y * v[kx + 1];
-                                a += g[j].z * v[kx + 2];
-                                a += g[j].w * v[kx + 3];
-                                acc[j][i][3 * ky + kx] = a;
-                            }
-                    }
-            }
+    };
+    stage(0, blockIdx.x);
+    for (int t = blockIdx.x, s = 0; t < A.ntiles; t += gridDim.x, s ^= 1) {
+        if (t + (int)gridDim.x < A.ntiles) {
+            stage(s ^ 1, t + gridDim.x);
+            cp_wait<1>();
+        } else {
+            cp_wait<0>();
         }
-        if (blockIdx.z == 0) {  // bias: BT neighbouring threads per channel
+        __syncthreads();
+        const float *tg = wg_sm + s * BUF, *tin = tg + COB * GP;
+#pragma unroll 1
+        for (int q = slice; q < TH * TS / 4; q += NS) {  // groups of four pixels
+            const int r = q / (TS / 4), x = (q % (TS / 4)) * 4;
+            float4 g[4];
+#pragma unroll
+            for (int j = 0; j < 4; j++)
+                g[j] = *reinterpret_cast<const float4 *>(tg + (cg + CG * j) * GP + r * TS + x);
+#pragma unroll
+            for (int i = 0; i < 2; i++)
+#pragma unroll
+                for (int ky = 0; ky < 3; ky++) {
+                    const float *row = tin + (ig + IG * i) * IP + (r + ky) * IW + x;
+                    const float4 va = *reinterpret_cast<const float4 *>(row);
+                    const float2 vb = *reinterpret_cast<const float2 *>(row + 4);
+                    const float v[6] = {va.x, va.y, va.z, va.w, vb.x, vb.y};
+#pragma unroll
+                    for (int kx = 0; kx < 3; kx++)
+#pragma unroll
+                        for (int j = 0; j < 4; j++) {
+                            float a = acc[j][i][3 * ky + kx];
+                            a += g[j].x * v[kx];
+                            a += g[j].y * v[kx + 1];
+                            a += g[j].z * v[kx + 2];
+                            a += g[j].w * v[kx + 3];
+                            acc[j][i][3 * ky + kx] = a;
+                        }
+                }
+        }
+        if (blockIdx.z == 0 && threadIdx.x < COB * BT) {  // bias: BT neighbouring threads per channel
             const float *g = tg + (threadIdx.x / BT) * GP;
-            for (int q = (threadIdx.x % BT) * 4; q < TS * TS; q += BT * 4) {
+            for (int q = (threadIdx.x % BT) * 4; q < TH * TS; q += BT * 4) {
                 const float4 v = *reinterpret_cast<const float4 *>(g + q);
                 bsum += (v.x + v.y) + (v.z + v.w);
             }
@@ -246,7 +296,7 @@ __global__ void __launch_bounds__(WG_T, 2)
                 wg_sm[(slice * 72 + (j * 2 + i) * 9 + k) * PT + pt] = acc[j][i][k];
     __syncthreads();
     const int nw = Cout * Cin * 9;
-    float *dst = part + (long)blockIdx.x * (nw + Cout);
+    float *dst = A.part + (long)blockIdx.x * (nw + Cout);
     for (int e = threadIdx.x; e < COB * CIB * 9; e += WG_T) {
         const int c = e / (CIB * 9), d = (e / 9) % CIB, k = e % 9;  // channels c, d of the block
         if (co0 + c < Cout && ci0 + d < Cin) {
@@ -259,9 +309,9 @@ __global__ void __launch_bounds__(WG_T, 2)
     }
     if (blockIdx.z == 0) {
 #pragma unroll
-        for (int o = (BT < 32 ? BT : 32) / 2; o > 0; o >>= 1) bsum += __shfl_down_sync(0xffffffffu, bsum, o, BT < 32 ? BT : 32);
+        for (int o = BT / 2; o > 0; o >>= 1) bsum += __shfl_down_sync(0xffffffffu, bsum, o, BT);
         const int c = threadIdx.x / BT;
-        if (threadIdx.x % BT == 0 && co0 + c < Cout) dst[nw + co0 + c] = bsum;
+        if (threadIdx.x < COB * BT && threadIdx.x % BT == 0 && co0 + c < Cout) dst[nw + co0 + c] = bsum;
     }
 }
 
@@ -516,6 +566,72 @@ __global__ void k_deflate_update(const double *__restrict__ info, const float *_
 
 int ck() { return cudaGetLastError() == cudaSuccess ? FEWHA_OK : FEWHA_ERR_CUDA; }
 
+// One launch of k_conv3x3, group by group.
+struct ConvLaunch {
+    ConvArgs A{};
+    long blocks = 0;
+    ConvLaunch(const float *w, const float *bias, int Cin, int Cout, int relu, int wt_mode)
+    {
+        A.w = w, A.bias = bias, A.Cin = Cin, A.Cout = Cout, A.relu = relu, A.wt_mode = wt_mode;
+    }
+    bool add(const float *in, long in_bs, long in_cs, float *out, long out_bs, long out_cs, const float *mask, int B,
+             int H, int W)
+    {
+        const int tx = (W + TX - 1) / TX, ty = (H + TY - 1) / TY;
+        const long z = (long)B * ((A.Cout + CO_T - 1) / CO_T), tiles = (long)tx * ty;
+        if (z > 65535 || tiles > 0x7FFFFFFFL || blocks + z * tiles > 0x7FFFFFFFL) return false;
+        A.g[A.ng++] = ConvGroup{in, mask, out, in_bs, in_cs, out_bs, out_cs, H, W, tx, (int)tiles, (int)blocks};
+        blocks += z * tiles;
+        return true;
+    }
+    int run(cudaStream_t s) const
+    {
+        k_conv3x3<<<(unsigned)blocks, NT, 0, s>>>(A);
+        return ck();
+    }
+};
+
+// One weight gradient: partials over the tiles of all groups, then their sum.
+struct WgradLaunch {
+    WgradArgs A{};
+    long ntiles = 0, parts = 0;  // parts: workspace capacity, TS x TS tiles
+    WgradLaunch(int Cin, int Cout) { A.Cin = Cin, A.Cout = Cout; }
+    bool add(const float *in, long in_bs, long in_cs, const float *gout, long gout_bs, long gout_cs, int B, int H, int W)
+    {
+        const long tx = (W + TS - 1) / TS, tiles = tx * ((H + TH - 1) / TH);
+        if (ntiles + tiles * B > 0x7fffffffL) return false;
+        A.g[A.ng++] = WgradGroup{in, gout, in_bs, in_cs, gout_bs, gout_cs, H, W, (int)tx, (int)tiles, (int)ntiles};
+        ntiles += tiles * B;
+        parts += tx * ((H + TS - 1) / TS) * B;
+        return true;
+    }
+    template <class K>
+    int partials(K kern, size_t bytes, int cob, int cib, int n, cudaStream_t s)
+    {
+        const dim3 grid(n, (A.Cout + cob - 1) / cob, (A.Cin + cib - 1) / cib);
+        if (grid.y > 65535 || grid.z > 65535) return FEWHA_ERR_ARG;
+        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess)
+            return FEWHA_ERR_CUDA;
+        kern<<<grid, WG_T, bytes, s>>>(A);
+        return ck();
+    }
+    int run(float *gw, float *gb, int accumulate, float *workspace, cudaStream_t s)
+    {
+        const int n = (int)(parts < WG_CTAS ? parts : WG_CTAS), Cin = A.Cin, Cout = A.Cout;  // n <= ntiles
+        A.part = workspace;
+        A.ntiles = (int)ntiles;
+        // channel block: 32 x 32, or narrow on the side with at most 8 output / 4
+        // input channels (the padding would be most of the work)
+        const int st = Cout <= 8  ? partials(k_conv3x3_wgrad_partial<2, 16>, wg_smem<2, 16>(), 8, 32, n, s)
+                       : Cin <= 4 ? partials(k_conv3x3_wgrad_partial<8, 2>, wg_smem<8, 2>(), 32, 4, n, s)
+                                  : partials(k_conv3x3_wgrad_partial<8, 16>, wg_smem<8, 16>(), 32, 32, n, s);
+        if (st != FEWHA_OK) return st;
+        const int len = Cout * Cin * 9 + Cout;
+        k_reduce_partials<<<(len + 31) / 32, 32 * RG, 0, s>>>(workspace, n, len, gw, gb, Cout * Cin * 9, accumulate);
+        return ck();
+    }
+};
+
 }  // namespace
 
 extern "C" {
@@ -524,11 +640,9 @@ int fewha_conv3x3_fwd(const float *in, long in_bs, long in_cs, int Cin, const fl
                       float *out, long out_bs, long out_cs, int Cout, int B, int H, int W, int relu, cudaStream_t s)
 {
     if (!in || !w || !out || Cin < 1 || Cout < 1 || B < 1 || H < 1 || W < 1) return FEWHA_ERR_ARG;
-    dim3 grid((W + TX - 1) / TX, (H + TY - 1) / TY, B * ((Cout + CO_T - 1) / CO_T));
-    if (grid.z > 65535) return FEWHA_ERR_ARG;
-    k_conv3x3<<<grid, NT, 0, s>>>(in, in_bs, in_cs, Cin, w, bias, out, out_bs, out_cs, Cout, H, W, relu, 0,
-                                    nullptr);
-    return ck();
+    ConvLaunch L(w, bias, Cin, Cout, relu, 0);
+    if (!L.add(in, in_bs, in_cs, out, out_bs, out_cs, nullptr, B, H, W)) return FEWHA_ERR_ARG;
+    return L.run(s);
 }
 
 int fewha_conv3x3_bwd_data_relu(const float *gout, long gout_bs, long gout_cs, int Cout, const float *w,
@@ -536,11 +650,9 @@ int fewha_conv3x3_bwd_data_relu(const float *gout, long gout_bs, long gout_cs, i
                                 cudaStream_t s)
 {
     if (!gout || !w || !gin || Cin < 1 || Cout < 1 || B < 1 || H < 1 || W < 1) return FEWHA_ERR_ARG;
-    dim3 grid((W + TX - 1) / TX, (H + TY - 1) / TY, B * ((Cin + CO_T - 1) / CO_T));
-    if (grid.z > 65535) return FEWHA_ERR_ARG;
-    k_conv3x3<<<grid, NT, 0, s>>>(gout, gout_bs, gout_cs, Cout, w, nullptr, gin, gin_bs, gin_cs, Cin, H, W, 0, 1,
-                                  act);
-    return ck();
+    ConvLaunch L(w, nullptr, Cout, Cin, 0, 1);
+    if (!L.add(gout, gout_bs, gout_cs, gin, gin_bs, gin_cs, act, B, H, W)) return FEWHA_ERR_ARG;
+    return L.run(s);
 }
 
 int fewha_conv3x3_bwd_data(const float *gout, long gout_bs, long gout_cs, int Cout, const float *w, float *gin,
@@ -565,25 +677,67 @@ int fewha_conv3x3_bwd_weight(const float *in, long in_bs, long in_cs, int Cin, c
     const long tiles = (long)((W + TS - 1) / TS) * ((H + TS - 1) / TS) * B;
     const size_t smem = ((size_t)Cin * (TS + 2) * (TS + 2) + (size_t)Cout * TS * TS) * sizeof(float);
     if (smem > 200 * 1024 || tiles > 0x7fffffffL) return FEWHA_ERR_ARG;
-    // channel block: 32 x 32, or narrow on the side with at most 8 output / 4
-    // input channels (the padding would be most of the work)
-    const int nparts = (int)(tiles < WG_CTAS ? tiles : WG_CTAS);
-    auto launch = [&](auto kern, size_t bytes, int cob, int cib) -> int {
-        const dim3 grid(nparts, (Cout + cob - 1) / cob, (Cin + cib - 1) / cib);
-        if (grid.y > 65535 || grid.z > 65535) return FEWHA_ERR_ARG;
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess)
-            return FEWHA_ERR_CUDA;
-        kern<<<grid, WG_T, bytes, s>>>(in, in_bs, in_cs, Cin, gout, gout_bs, gout_cs, Cout, H, W, (int)tiles,
-                                       workspace);
-        return ck();
-    };
-    const int st = Cout <= 8  ? launch(k_conv3x3_wgrad_partial<2, 16>, wg_smem<2, 16>(), 8, 32)
-                   : Cin <= 4 ? launch(k_conv3x3_wgrad_partial<8, 2>, wg_smem<8, 2>(), 32, 4)
-                              : launch(k_conv3x3_wgrad_partial<8, 16>, wg_smem<8, 16>(), 32, 32);
-    if (st != FEWHA_OK) return st;
-    const int len = Cout * Cin * 9 + Cout;
-    k_reduce_partials<<<(len + 31) / 32, 32 * RG, 0, s>>>(workspace, nparts, len, gw, gb, Cout * Cin * 9, accumulate);
-    return ck();
+    WgradLaunch L(Cin, Cout);
+    if (!L.add(in, in_bs, in_cs, gout, gout_bs, gout_cs, B, H, W)) return FEWHA_ERR_ARG;
+    return L.run(gw, gb, accumulate, workspace, s);
+}
+
+// The training network (C0 -> C -> C -> C3, ReLU after the first two) over groups
+// of equal-size images: image i of group g starts off[g] + i side[g]^2 floats
+// into a channel of x, y and gy; the hidden activations and their gradients are
+// (count[g], C, side, side) arrays of their own.
+static int net_args_ok(const fewha_net *N)
+{
+    if (!N || N->ngroups < 1 || N->ngroups > kMaxGroups || N->C0 < 1 || N->C < 1 || N->C3 < 1) return 0;
+    for (int i = 0; i < 3; i++)
+        if (!N->w[i] || !N->b[i]) return 0;
+    for (int g = 0; g < N->ngroups; g++)
+        if (N->count[g] < 1 || N->side[g] < 1 || N->off[g] < 0 || !N->h1[g] || !N->h2[g]) return 0;
+    return 1;
+}
+
+int fewha_convnet_fwd(const fewha_net *N, const float *x, long x_cs, float *y, long y_cs, cudaStream_t s)
+{
+    if (!net_args_ok(N) || !x || !y) return FEWHA_ERR_ARG;
+    ConvLaunch L1(N->w[0], N->b[0], N->C0, N->C, 1, 0), L2(N->w[1], N->b[1], N->C, N->C, 1, 0),
+        L3(N->w[2], N->b[2], N->C, N->C3, 0, 0);
+    for (int g = 0; g < N->ngroups; g++) {
+        const int B = N->count[g], S = N->side[g];
+        const long hw = (long)S * S, hb = N->C * hw;
+        if (!L1.add(x + N->off[g], hw, x_cs, N->h1[g], hb, hw, nullptr, B, S, S) ||
+            !L2.add(N->h1[g], hb, hw, N->h2[g], hb, hw, nullptr, B, S, S) ||
+            !L3.add(N->h2[g], hb, hw, y + N->off[g], hw, y_cs, nullptr, B, S, S))
+            return FEWHA_ERR_ARG;
+    }
+    int st = L1.run(s);
+    if (st == FEWHA_OK) st = L2.run(s);
+    return st == FEWHA_OK ? L3.run(s) : st;
+}
+
+int fewha_convnet_bwd(const fewha_net *N, const float *x, long x_cs, const float *gy, long gy_cs, float *workspace,
+                      cudaStream_t s)
+{
+    if (!net_args_ok(N) || !x || !gy || !workspace) return FEWHA_ERR_ARG;
+    for (int i = 0; i < 3; i++)
+        if (!N->gw[i] || !N->gb[i]) return FEWHA_ERR_ARG;
+    WgradLaunch W1(N->C0, N->C), W2(N->C, N->C), W3(N->C, N->C3);
+    ConvLaunch D3(N->w[2], nullptr, N->C3, N->C, 0, 1), D2(N->w[1], nullptr, N->C, N->C, 0, 1);
+    for (int g = 0; g < N->ngroups; g++) {
+        if (!N->g1[g] || !N->g2[g]) return FEWHA_ERR_ARG;
+        const int B = N->count[g], S = N->side[g];
+        const long hw = (long)S * S, hb = N->C * hw;
+        const float *xg = x + N->off[g], *gg = gy + N->off[g];
+        if (!W3.add(N->h2[g], hb, hw, gg, hw, gy_cs, B, S, S) || !W2.add(N->h1[g], hb, hw, N->g2[g], hb, hw, B, S, S) ||
+            !W1.add(xg, hw, x_cs, N->g1[g], hb, hw, B, S, S) ||
+            !D3.add(gg, hw, gy_cs, N->g2[g], hb, hw, N->h2[g], B, S, S) ||
+            !D2.add(N->g2[g], hb, hw, N->g1[g], hb, hw, N->h1[g], B, S, S))
+            return FEWHA_ERR_ARG;
+    }
+    int st = W3.run(N->gw[2], N->gb[2], 0, workspace, s);
+    if (st == FEWHA_OK) st = D3.run(s);
+    if (st == FEWHA_OK) st = W2.run(N->gw[1], N->gb[1], 0, workspace, s);
+    if (st == FEWHA_OK) st = D2.run(s);
+    return st == FEWHA_OK ? W1.run(N->gw[0], N->gb[0], 0, workspace, s) : st;
 }
 
 int fewha_relu_bwd(const float *act, float *g, long n, cudaStream_t s)

@@ -59,6 +59,14 @@ class OPTS(C.Structure):
                 ("rhs_in_state", C.c_int), ("pad", C.c_int), ("c_out", C.c_void_p)]
 
 
+class NET(C.Structure):
+    """fewha_net: the training network's groups and buffers."""
+    _fields_ = [("C0", C.c_int), ("C", C.c_int), ("C3", C.c_int), ("ngroups", C.c_int), ("count", C.c_int * 8),
+                ("side", C.c_int * 8), ("off", C.c_long * 8), ("h1", C.c_void_p * 8), ("h2", C.c_void_p * 8),
+                ("g1", C.c_void_p * 8), ("g2", C.c_void_p * 8), ("w", C.c_void_p * 3), ("b", C.c_void_p * 3),
+                ("gw", C.c_void_p * 3), ("gb", C.c_void_p * 3)]
+
+
 class LAUNCH_INFO(C.Structure):
     _fields_ = [("ctas", C.c_int), ("threads", C.c_int), ("smem_bytes", C.c_long),
                 ("split_levels", C.c_int), ("staged_tables", C.c_int), ("wfs_tile_y", C.c_int),
@@ -159,6 +167,8 @@ def load_library(path=LIB_PATH):
     learned = {
         "fewha_conv3x3_fwd": [vp, L, L, I, vp, vp, vp, L, L, I, I, I, I, I, vp],
         "fewha_conv3x3_fwd_tc": [vp, L, L, I, vp, vp, vp, L, L, I, I, I, I, I, vp, vp],
+        "fewha_convnet_fwd": [C.POINTER(NET), vp, L, vp, L, vp],
+        "fewha_convnet_bwd": [C.POINTER(NET), vp, L, vp, L, vp, vp],
         "fewha_convnet_fwd_tc": [vp, L, I, vp, vp, vp, vp, vp, vp, vp, L, I, I, C.POINTER(C.c_int),
                                  C.POINTER(C.c_int), C.POINTER(C.c_long), vp, vp],
         "fewha_conv3x3_bwd_data_relu": [vp, L, L, I, vp, vp, vp, L, L, I, I, I, I, vp],
@@ -198,7 +208,8 @@ def exported_symbols():
             "fewha_mse_grad", "fewha_adam_step", "fewha_scale", "fewha_learned_targets",
             "fewha_deflate_warm_start", "fewha_mcao_create", "fewha_mcao_n_actuators", "fewha_mcao_fit",
             "fewha_mcao_destroy", "fewha_get_launch_info", "fewha_set_noise", "fewha_read_probe", "fewha_set_pt_bands",
-            "fewha_batch_create_ex", "fewha_batch_tiles", "fewha_conv3x3_fwd_tc", "fewha_convnet_fwd_tc", "fewha_store"]
+            "fewha_batch_create_ex", "fewha_batch_tiles", "fewha_conv3x3_fwd_tc", "fewha_convnet_fwd_tc", "fewha_convnet_fwd",
+            "fewha_convnet_bwd", "fewha_store"]
 
 
 def make_geometry(geom, noise_w, precision="f64", tile=0, grid=0) -> GEOMETRY:

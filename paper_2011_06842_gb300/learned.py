@@ -27,7 +27,7 @@ import math
 
 import numpy as np
 
-from .fewha import FewhaError, _stream_ptr, load_library
+from .fewha import NET, FewhaError, _stream_ptr, load_library
 
 CHANNELS = (4, 32, 32, 5)
 TC_MAX_GROUPS = 8  # most layer sizes of one launch of the whole network
@@ -105,6 +105,10 @@ class ConvNet:
         self._tc_groups = ((C.c_int * ng)(*[cnt for _, cnt, _ in self.groups]),
                            (C.c_int * ng)(*[nl for _, _, nl in self.groups]),
                            (C.c_long * ng)(*[off for off, _, _ in self.groups]))
+        # every group's partial sums of a weight gradient in one launch
+        tiles = sum(cnt * ((nl + 15) // 16) ** 2 for _, cnt, nl in self.groups)
+        ws = max(ws, min(152, tiles) * (9 * c1 * max(c0, c2, c3) + max(c1, c2, c3)))
+        self._net = None
         self._hidden = True  # h1, h2 hold the activations of the last forward()
         self.work = torch.empty(max(ws, 1), dtype=torch.float32, device=dev)
         self.loss_part = torch.zeros(512, dtype=torch.float64, device=dev)
@@ -134,9 +138,31 @@ class ConvNet:
             self._hidden = False
             return y
         self._hidden = True
+        if not tensor_cores and len(self.groups) <= TC_MAX_GROUPS:
+            self._ck(self.lib.fewha_convnet_fwd(C.byref(self._net_args()), C.c_void_p(x_ptr), x_cs,
+                                                C.c_void_p(y.data_ptr()), y.stride(0), _stream_ptr(self.torch)),
+                     "convnet")
+            return y
         for name, _, launch in self.convolutions(x_ptr, x_cs, y, tensor_cores):
             self._ck(launch(), name)
         return y
+
+    def _net_args(self):
+        """The network's buffers for fewha_convnet_fwd and _bwd (they live as long as this object)."""
+        if self._net is None:
+            N = self._net = NET()
+            N.C0, N.C, _, N.C3 = CHANNELS
+            N.ngroups = len(self.groups)
+            for g, (off, cnt, nl) in enumerate(self.groups):
+                N.count[g], N.side[g], N.off[g] = cnt, nl, off
+                N.h1[g], N.h2[g] = self.h1[g].data_ptr(), self.h2[g].data_ptr()
+                N.g2[g], N.g1[g] = self.ga[g].data_ptr(), self.gb[g].data_ptr()
+        N = self._net
+        for i in range(3):
+            for dst, src, k in ((N.w, self.param, "w"), (N.b, self.param, "b"), (N.gw, self.grad, "w"),
+                                (N.gb, self.grad, "b")):
+                dst[i] = self._p(src, k + str(i + 1)).value
+        return N
 
     def _tc_status(self):
         if not hasattr(self, "tc_status"):
@@ -181,6 +207,10 @@ class ConvNet:
                 if i % 3 < 2:  # the two hidden layers of each group
                     self._ck(launch(), name)
             self._hidden = True
+        if len(self.groups) <= TC_MAX_GROUPS:
+            self._ck(lib.fewha_convnet_bwd(C.byref(self._net_args()), C.c_void_p(x_ptr), x_cs,
+                                           C.c_void_p(gy.data_ptr()), gy.stride(0), work, s), "convnet backward")
+            return
         for gi, (off, cnt, nl) in enumerate(self.groups):
             hw = nl * nl
             acc = 1 if gi > 0 else 0
