@@ -612,6 +612,8 @@ struct ImplBase {
     // WFS tile shape for a group of `ctas` CTAs, and the dynamic shared memory it needs
     virtual int tiles_for(int ctas, int *ty, int *tx) const = 0;
     virtual size_t smem_for(int ty, int tx) const = 0;
+    // the same, with what a faster plan for small groups needs (at creation of a batch)
+    virtual size_t smem_want(int ty, int tx) const = 0;
     // host copy of this instance's kernel arguments for one time step
     virtual int batch_args(void *out, const void *sl, void *c, const fewha_state *st, const fewha_solve_opts *o,
                            fewha_stats *stats, int cta0, int ncta, int ty, int tx, size_t smem) const = 0;
@@ -639,6 +641,7 @@ struct Impl : ImplBase {
     unsigned char *multi_buf = nullptr;  // scratch of apply_multi (allocated on first use)
     size_t multi_stride = 0;
 
+    static constexpr int kBandLarge = 8, kBandSmall = 4;  // default P^T band heights (plan_bands)
     size_t sm_fixed = 0;  // dynamic shared memory of every phase but the WFS tiles
     size_t sm_base = 0;   // of the layer and WFS phases alone (before the P^T bands)
     size_t sm_layer_ = 0; // of the layer phases alone
@@ -646,6 +649,13 @@ struct Impl : ImplBase {
     size_t ll_elems() const { return (size_t)P.n / 4 + P.n / 16 + 1; }  // Args::ll
     std::vector<void *> band_owned;  // device tables of the P^T bands (replaced by plan_bands)
     int band_rows_large = 0, band_rows_small = 0;
+    // second P^T band plan, for groups with several bands per CTA: the tallest
+    // bands (kBandOutputs outputs each).  A band takes a CTA about 7 us whatever its
+    // size (staging and contraction latencies), so fewer rounds of bands are
+    // faster: 9 ELT layers on 9 CTAs take 16 rounds of 8- and 4-row bands.
+    Geo<T> few{};
+    std::vector<void *> few_owned;
+    size_t few_fixed = 0;  // its sm_fixed; 0: no such plan
 
     explicit Impl(const Plan &p) : P(p) {}
 
@@ -695,6 +705,29 @@ struct Impl : ImplBase {
     }
 
     size_t smem_for(int ty, int tx) const override { return std::max(sm_fixed, wfs_bytes(ty, tx)); }
+    // with room for the second band plan
+    size_t smem_want(int ty, int tx) const override
+    {
+        return std::max(smem_for(ty, tx), few_usable() ? few_fixed : 0);
+    }
+
+    // band heights that a caller set explicitly (set_bands) hold for every group
+    bool few_usable() const { return few_fixed > 0 && band_rows_large == kBandLarge && band_rows_small == kBandSmall; }
+
+    // the P^T band plan for a group of nct CTAs with sm bytes of shared memory:
+    // the one with fewer rounds
+    void choose_bands(Geo<T> &G, int nct, size_t sm) const
+    {
+        auto rounds = [&](int nb) { return (nb + nct - 1) / nct; };
+        if (!few_usable() || few_fixed > sm || rounds(few.nbands) >= rounds(G.nbands)) return;
+        G.nbands = few.nbands;
+        G.band_layer = few.band_layer, G.band_row0 = few.band_row0, G.band_rows = few.band_rows;
+        G.band_ilo = few.band_ilo, G.band_ihi = few.band_ihi;
+        G.band_gend = few.band_gend, G.band_gc = few.band_gc, G.band_gr = few.band_gr;
+        G.rows_chunk = few.rows_chunk, G.stage_tab = few.stage_tab;
+        G.band_ycnt = few.band_ycnt, G.band_yrow = few.band_yrow, G.band_yw = few.band_yw;
+        G.ybr = few.ybr, G.ymax = few.ymax;
+    }
     size_t args_size() const override { return sizeof(Args<T, S>); }
     int precision_id() const override
     {
@@ -704,6 +737,7 @@ struct Impl : ImplBase {
     {
         for (void *q : owned) cudaFree(q);
         for (void *q : band_owned) cudaFree(q);
+        for (void *q : few_owned) cudaFree(q);
     }
 
     template <typename U>
@@ -1018,7 +1052,14 @@ struct Impl : ImplBase {
         smem = std::max(sm_layer, sm_wfs);
         sm_base = smem;
         sm_layer_ = sm_layer;
-        if ((st = plan_bands(8, 4))) return st;
+        if ((st = plan_bands(FEWHA_MAX_GRID, FEWHA_MAX_GRID)) == FEWHA_OK) {
+            few = G;
+            few_owned.swap(band_owned);
+            few_fixed = sm_fixed;
+        } else if (st != FEWHA_ERR_GEOMETRY) {
+            return st;  // (too many rows for the shared memory: no second plan)
+        }
+        if ((st = plan_bands(kBandLarge, kBandSmall))) return st;
         int dev, nsm;
         CK(cudaGetDevice(&dev));
         CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
@@ -1471,7 +1512,7 @@ struct Impl : ImplBase {
         const int per = std::max(1, ncta / nvec);
         int ty, tx;
         if (tiles_for(per, &ty, &tx)) return FEWHA_ERR_GEOMETRY;
-        const size_t sm = smem_for(ty, tx);
+        const size_t sm = smem_want(ty, tx);
         MultiArgs<T, S> M{};
         M.per = per;
         for (int v = 0; v < nvec; v++) {
@@ -1487,6 +1528,7 @@ struct Impl : ImplBase {
             A.cta0 = v * per;
             A.ncta = per;
             set_tiles(A.geo, ty, tx);
+            choose_bands(A.geo, per, sm);
             A.smem_bytes = sm;
             A.trace = nullptr;
             A.trace_cap = 0;
@@ -1573,6 +1615,7 @@ struct Impl : ImplBase {
         A.cta0 = cta0;
         A.ncta = nct;
         set_tiles(A.geo, ty, tx);
+        choose_bands(A.geo, nct, sm);
         A.smem_bytes = sm;
         A.trace = nullptr;
         A.trace_cap = 0;
