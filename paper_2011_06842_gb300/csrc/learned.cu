@@ -47,7 +47,9 @@ constexpr int TP = TX + 4;  // pitch of a staged row: x0-1 .. x0+TX plus slack, 
 // (16-byte loads, the same for every lane), 36 shared-memory wavefronts for 288
 // FMAs per thread, against 60 for 288 with two vertically adjacent pixels and
 // single loads.  Input tiles and weights of the next CI_T channels are copied
-// asynchronously while the present ones are used.
+// asynchronously while the present ones are used.  32 -> 32 channels over 5 x
+// 128^2 and 4 x 64^2 pixels: 76 us in one launch (79 + 24 us in two of eight staged
+// channels and four CTAs per SM).
 //
 // A launch covers up to kMaxGroups groups of equal-size images (the layers of
 // each size): a group of small images alone leaves most SMs idle.
@@ -171,7 +173,7 @@ __global__ void __launch_bounds__(NT, CONV_CTAS) k_conv3x3(const __grid_constant
 // for every FMA).  The slices are summed in slice order at the end.  With the
 // parallel sum of the partials below and the four-pixel convolution above, a
 // training step on the ELT layers (5 x 128^2 and 4 x 64^2) went from 1171 to
-// 596 us.
+// 596 us; with the groups in one launch and 152 CTAs, to 418 us.
 constexpr int TS = 16;           // width of the spatial tile; the workspace counts TS x TS tiles
 constexpr int TH = 8;            // its height: 16 x 8 tiles spread over the CTAs more evenly than 16 x 16
 constexpr int WG_T = 512;        // threads

@@ -251,10 +251,10 @@ __device__ __forceinline__ void phase_init(const Args<T, S> &A, const Basis &b, 
 // ---------------------------------------------------------------------------
 // Finest levels that the split form tiles over all CTAs: one, or two in FP64
 // with layers of at least 128^2 (Geo::depth, set on the host).  A layer CTA has
-// about two FP64 FMAs per clock: the 64^2 block of a 128^2 layer keeps it ~26 us
-// in UA1 and again in D2E (8 operations per element of the update, 12 per
-// element and level of the transform), the 32^2 block a quarter of that, for one
-// more tiled phase and barrier on each side.  In FP32 the block is latency
+// about two FP64 FMAs per clock (8 operations per element of the update, 12 per
+// element and level of the transform): with the 64^2 block of a 128^2 layer UA1
+// took 57 us and D2E 45, with the 32^2 block 26 and 22 (15 and 13.5 with the runs
+// of dwt_pass), for one more tiled phase and barrier on each side (3.7 + 1 us).  In FP32 the block is latency
 // bound and a phase with its barrier costs more than the level saves.
 template <typename T>
 __device__ __forceinline__ int split_depth(const Geo<T> &G)
