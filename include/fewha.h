@@ -512,7 +512,8 @@ void fewha_mcao_destroy(void *mcao);
  * device (no cached pointer outlives a device reset); the current device must
  * be the handle's (FEWHA_ERR_ARG otherwise).  Problems whose buffers do not
  * fit are rejected with FEWHA_ERR_SCRATCH (an ELT-size FP64 operator, n =
- * 98304 with 6 sensors of 84 x 84 subapertures, needs about 4.8 MB).
+ * 98304 with 6 sensors of 84 x 84 subapertures, counts as about 4.8 MB, of
+ * which 3 MB are reserved for partial sums).
  * All calls share the one array, which keeps the last call's contents: calls
  * that overlap on the GPU (different streams, different handles on the same
  * device) race and must be ordered by the caller.  The paper has no
