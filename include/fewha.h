@@ -35,6 +35,10 @@
  *    [x slopes | y slopes], each n_g x n_g row-major (row = y).  Entries of
  *    unlit subapertures are ignored.
  *  - Asynchrony: compute calls enqueue work on the given stream and return.
+ *    Calls on one handle share its scratch memory, so those that overlap on
+ *    the GPU (different streams) must be ordered by the caller.  Exception:
+ *    fewha_rhs may overlap fewha_fit and fewha_mcao_fit (the next frame's
+ *    right-hand side beside this frame's fitting).
  */
 #ifndef FEWHA_H
 #define FEWHA_H

@@ -649,6 +649,9 @@ struct Impl : ImplBase {
     size_t sm_layer_ = 0; // of the layer phases alone
     size_t sm_fine_ = 0;  // of the tiled wavelet levels alone
     size_t ll_elems() const { return (size_t)P.n / 4 + P.n / 16 + 1; }  // Args::ll
+    // Args::ll of W^{-1} c (fit, mcao_fit).  A loop may fit one frame while it forms the
+    // next right-hand side on another stream of the same handle: the two calls write no buffer in common.
+    T *ll_nodal = nullptr;
     std::vector<void *> band_owned;  // device tables of the P^T bands (replaced by plan_bands)
     int band_rows_large = 0, band_rows_small = 0;
     // second P^T band plan, for groups with several bands per CTA: the tallest
@@ -1023,7 +1026,8 @@ struct Impl : ImplBase {
         if ((st = alloc((size_t)P.n, &base.nodal)) || (st = alloc((size_t)P.n, &base.u)) ||
             (st = alloc((size_t)P.n, &base.wq)) ||
             (st = alloc((size_t)P.psi_off[P.G], &base.psi)) || (st = alloc(ll_elems(), &base.ll)) ||
-            (st = alloc((size_t)kSlots * kMaxCtas, &base.part)) || (st = alloc((size_t)1, &base.rec)))
+            (st = alloc(ll_elems(), &ll_nodal)) || (st = alloc((size_t)kSlots * kMaxCtas, &base.part)) ||
+            (st = alloc((size_t)1, &base.rec)))
             return st;
         if constexpr (std::is_same<T, S>::value) {
             base.nodal_t = base.nodal;
@@ -1288,6 +1292,7 @@ struct Impl : ImplBase {
     {
         Args<T, S> A = base;
         A.x = static_cast<const T *>(c);
+        A.ll = ll_nodal;
         OpChain run{ncta, s, true, cudaSuccess};
         op_idwt(run, A, ncta, smem);
         return run.err == cudaSuccess ? FEWHA_OK : FEWHA_ERR_CUDA;
