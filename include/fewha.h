@@ -421,7 +421,8 @@ int fewha_convnet_bwd(const fewha_net *net, const float *x, long x_cs, const flo
  *   fewha_conv3x3_fwd_tc calls; C0, C3 <= 16.  Image i of group g (count[g]
  *   images of side[g] x side[g], side <= 128; at most 8 groups; host arrays)
  *   starts off[g] + i side[g]^2 floats into a channel of in and out; in_cs and
- *   out_cs are the channel strides.  status_dev as in fewha_conv3x3_fwd_tc. */
+ *   out_cs are the channel strides; out must not overlap in.  status_dev as in
+ *   fewha_conv3x3_fwd_tc. */
 int fewha_convnet_fwd_tc(const float *in, long in_cs, int C0, const float *w1, const float *b1, const float *w2,
                          const float *b2, const float *w3, const float *b3, float *out, long out_cs, int C3,
                          int ngroups, const int *count, const int *side, const long *off, int *status_dev,

@@ -63,6 +63,13 @@ def scale_groups(geom):
     return np.concatenate(out).astype(np.int8)
 
 
+def _overlap(x_ptr, x_cs, cx, y_ptr, y_cs, cy, n):
+    """Whether the spans of cx and cy FP32 channels of n values (strides x_cs, y_cs) may share memory."""
+    ex, ey = (cx - 1) * x_cs, (cy - 1) * y_cs
+    return (x_ptr + 4 * min(ex, 0) < y_ptr + 4 * (max(ey, 0) + n)
+            and y_ptr + 4 * min(ey, 0) < x_ptr + 4 * (max(ex, 0) + n))
+
+
 class ConvNet:
     """Parameters, Adam state and activation buffers of the network on the GPU."""
 
@@ -127,9 +134,12 @@ class ConvNet:
         operands, FP32 accumulation; inference), else on the FP32 kernel
         (training: its activations feed the backward pass).  On the tensor
         cores the whole network is one launch that keeps the hidden layers on
-        chip; backward() forms them again."""
-        if tensor_cores and len(self.groups) <= TC_MAX_GROUPS:
-            c0, _, _, c3 = CHANNELS
+        chip; backward() forms them again.  y may lie over x (its memory then
+        holds y): the network then runs layer by layer, because a block of that
+        launch reads input rows beside those whose outputs another block writes."""
+        c0, _, _, c3 = CHANNELS
+        if tensor_cores and len(self.groups) <= TC_MAX_GROUPS and not _overlap(x_ptr, x_cs, c0, y.data_ptr(),
+                                                                               y.stride(0), c3, self.n):
             p = lambda k: self._p(self.param, k)  # noqa: E731
             self._ck(self.lib.fewha_convnet_fwd_tc(C.c_void_p(x_ptr), x_cs, c0, p("w1"), p("b1"), p("w2"), p("b2"),
                                                    p("w3"), p("b3"), C.c_void_p(y.data_ptr()), y.stride(0), c3,
