@@ -116,7 +116,7 @@ class ConvNet:
         tiles = sum(cnt * ((nl + 15) // 16) ** 2 for _, cnt, nl in self.groups)
         ws = max(ws, min(152, tiles) * (9 * c1 * max(c0, c2, c3) + max(c1, c2, c3)))
         self._net = None
-        self._hidden = True  # h1, h2 hold the activations of the last forward()
+        self._hidden = True  # the last forward() left its hidden layers in h1, h2
         self.work = torch.empty(max(ws, 1), dtype=torch.float32, device=dev)
         self.loss_part = torch.zeros(512, dtype=torch.float64, device=dev)
 
@@ -208,7 +208,9 @@ class ConvNet:
         return out
 
     def backward(self, x_ptr, x_cs, gy):
-        """Parameter gradients (self.grad) of sum(gy * y) after forward() on the same x."""
+        """Parameter gradients (self.grad) of sum(gy * y) after forward() on the same x.  After a
+        tensor-core forward() every call forms the hidden layers from x again: a replayed graph of
+        that forward leaves none behind."""
         lib, s = self.lib, _stream_ptr(self.torch)
         c0, c1, c2, c3 = CHANNELS
         work = C.c_void_p(self.work.data_ptr())
@@ -216,7 +218,6 @@ class ConvNet:
             for i, (name, _, launch) in enumerate(self.convolutions(x_ptr, x_cs, gy, tensor_cores=True)):
                 if i % 3 < 2:  # the two hidden layers of each group
                     self._ck(launch(), name)
-            self._hidden = True
         if len(self.groups) <= TC_MAX_GROUPS:
             self._ck(lib.fewha_convnet_bwd(C.byref(self._net_args()), C.c_void_p(x_ptr), x_cs,
                                            C.c_void_p(gy.data_ptr()), gy.stride(0), work, s), "convnet backward")

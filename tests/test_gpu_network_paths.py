@@ -37,3 +37,29 @@ def test_output_over_the_input(name, tensor_cores):
     both[1:].copy_(x.flip(0))
     net.forward(both[4].data_ptr(), -net.n, both, tensor_cores=tensor_cores)
     assert float((both - y).norm() / y.norm()) < 1e-4
+
+
+def test_backward_after_replays_of_a_captured_forward():
+    """A captured tensor-core forward replayed on new inputs, each followed by backward(): the gradients of the
+    same calls without a graph (the same launches, bit for bit)."""
+    net = network(configs.tiny())
+    g = torch.Generator(device="cuda").manual_seed(1)
+    xs = torch.randn(3, 4, net.n, generator=g, device="cuda")
+    gy = torch.randn(5, net.n, generator=g, device="cuda")
+    x, y = xs[0].clone(), torch.empty_like(gy)
+    net.forward(x.data_ptr(), net.n, y, tensor_cores=True)  # everything the call needs is loaded before the capture
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        net.forward(x.data_ptr(), net.n, y, tensor_cores=True)
+    replayed = []
+    for i in range(3):
+        x.copy_(xs[i])
+        graph.replay()
+        net.backward(x.data_ptr(), net.n, gy)
+        replayed.append(net.grad.clone())
+    for i in range(3):
+        x.copy_(xs[i])
+        net.forward(x.data_ptr(), net.n, y, tensor_cores=True)
+        net.backward(x.data_ptr(), net.n, gy)
+        assert torch.equal(replayed[i], net.grad), i
