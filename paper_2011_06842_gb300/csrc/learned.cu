@@ -164,7 +164,7 @@ __global__ void __launch_bounds__(NT, CONV_CTAS) k_conv3x3(const __grid_constant
 }
 
 // Partial weight/bias gradients.  A CTA takes spatial tiles of TS x TH pixels
-// (tile blockIdx.x, + gridDim.x, ...) and one block of 4 CG output times 2 IG
+// (tile t0 + blockIdx.x, + gridDim.x, ...) and one block of 4 CG output times 2 IG
 // input channels; the next tile's gradients and inputs are copied to shared
 // memory while the present one is used,
 // and a thread keeps 4 x 2 x 9 sums in registers for its slice of the tile's
@@ -178,6 +178,15 @@ constexpr int TS = 16;           // width of the spatial tile; the workspace cou
 constexpr int TH = 8;            // its height: 16 x 8 tiles spread over the CTAs more evenly than 16 x 16
 constexpr int WG_T = 512;        // threads
 constexpr int WG_CTAS = 152;     // CTAs of one launch, one per SM: the fewer, the fewer partials to add in FP64
+// Most tiles of one FP32 partial: a thread of the 32 x 32 block adds 32 products a
+// tile one after another, one of the narrow blocks 4 or 8 (and more slices at the
+// end), so that an FP32 sum is about as long as one 16 x 16 tile's 256 products,
+// whose error it is held to: against 64 bits, normal data, rms 2.1e-7 at the limit
+// (16 x 16 tiles 2.1e-7; without a limit 5.2e-7 at 54 tiles).  More tiles go in
+// rounds of WG_ROUND partials and one tile less each, whose FP64 sums are carried
+// from round to round in the rest of the workspace, 20 us a round.
+constexpr int WG_ROUND = WG_CTAS - 3;
+constexpr int wg_span(int slices) { return slices > 4 ? 24 : 8; }
 constexpr int GP = TH * TS + 4;  // channel pitch of the staged gradients: 8 channels on 8 different 16-byte banks
 constexpr int IW = TS + 4;       // row pitch of the staged inputs
 constexpr int IP = (TH + 2) * IW + 4;  // channel pitch of the staged inputs (odd multiple of 16 bytes)
@@ -190,7 +199,7 @@ struct WgradGroup {
 struct WgradArgs {
     WgradGroup g[kMaxGroups];
     float *part;
-    int ng, Cin, Cout, ntiles;
+    int ng, Cin, Cout, t0, t1;  // the launch's tiles t0 .. t1 - 1
 };
 
 template <int CG, int IG>
@@ -239,9 +248,9 @@ __global__ void __launch_bounds__(WG_T, 1) k_conv3x3_wgrad_partial(const __grid_
         }
         cp_commit();
     };
-    stage(0, blockIdx.x);
-    for (int t = blockIdx.x, s = 0; t < A.ntiles; t += gridDim.x, s ^= 1) {
-        if (t + (int)gridDim.x < A.ntiles) {
+    stage(0, A.t0 + blockIdx.x);
+    for (int t = A.t0 + blockIdx.x, s = 0; t < A.t1; t += gridDim.x, s ^= 1) {
+        if (t + (int)gridDim.x < A.t1) {
             stage(s ^ 1, t + gridDim.x);
             cp_wait<1>();
         } else {
@@ -318,14 +327,16 @@ __global__ void __launch_bounds__(WG_T, 1) k_conv3x3_wgrad_partial(const __grid_
 }
 
 // Sum of the CTAs' partials (deterministic, FP64); accumulate adds to the
-// gradients already stored.  32 outputs per CTA, RG threads each: thread g of
+// gradients already stored.  Rounds of partials: carry_in adds the totals of the
+// earlier ones, carry_out stores the totals instead of the gradients.  32 outputs per CTA, RG threads each: thread g of
 // an output sums partials g, g + RG, ..., then the RG sums are added in order.
 // One thread per output walked all partials with one load in flight.
 constexpr int RG = 8;
 
 __global__ void __launch_bounds__(32 * RG)
     k_reduce_partials(const float *__restrict__ part, int nparts, int len, float *__restrict__ gw,
-                      float *__restrict__ gb, int nw, int accumulate)
+                      float *__restrict__ gb, int nw, int accumulate, double *__restrict__ total, int carry_in,
+                      int carry_out)
 {
     __shared__ double sh[RG][32];
     const int lane = threadIdx.x & 31, g = threadIdx.x >> 5, e = blockIdx.x * 32 + lane;
@@ -345,6 +356,11 @@ __global__ void __launch_bounds__(32 * RG)
     if (g == 0 && e < len) {
 #pragma unroll
         for (int i = 1; i < RG; i++) a += sh[i][lane];
+        if (carry_in) a += total[e];
+        if (carry_out) {
+            total[e] = a;
+            return;
+        }
         float *dst = e < nw ? gw + e : gb + (e - nw);
         *dst = accumulate ? *dst + (float)a : (float)a;
     }
@@ -607,9 +623,12 @@ struct WgradLaunch {
         parts += tx * ((H + TS - 1) / TS) * B;
         return true;
     }
-    template <class K>
-    int partials(K kern, size_t bytes, int cob, int cib, int n, cudaStream_t s)
+    template <int CG, int IG>
+    int partials(int n, cudaStream_t s)
     {
+        auto kern = k_conv3x3_wgrad_partial<CG, IG>;
+        constexpr int cob = 4 * CG, cib = 2 * IG;
+        constexpr size_t bytes = wg_smem<CG, IG>();
         const dim3 grid(n, (A.Cout + cob - 1) / cob, (A.Cin + cib - 1) / cib);
         if (grid.y > 65535 || grid.z > 65535) return FEWHA_ERR_ARG;
         if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess)
@@ -617,20 +636,37 @@ struct WgradLaunch {
         kern<<<grid, WG_T, bytes, s>>>(A);
         return ck();
     }
+    template <int CG, int IG>
+    int gradient(float *gw, float *gb, int accumulate, float *workspace, cudaStream_t s)
+    {
+        constexpr int span = wg_span(WG_T / (CG * IG));
+        const int len = A.Cout * A.Cin * 9 + A.Cout;
+        const bool rounds = ntiles > (long)WG_CTAS * span;
+        // n <= ntiles.  With rounds the workspace holds WG_CTAS partials: the FP64
+        // totals (2 len floats and one for their alignment) lie behind the first n.
+        static_assert(WG_CTAS - WG_ROUND >= 3, "room for the totals");
+        const int n = rounds ? WG_ROUND : (int)(parts < WG_CTAS ? parts : WG_CTAS);
+        const long most = (long)n * (span - 1), nr = rounds ? (ntiles + most - 1) / most : 1;
+        double *total = reinterpret_cast<double *>((reinterpret_cast<size_t>(workspace + (long)n * len) + 7) & ~(size_t)7);
+        A.part = workspace;
+        for (long r = 0; r < nr; r++) {
+            A.t0 = (int)(r * ntiles / nr);  // rounds of equal size, n < tiles <= most
+            A.t1 = (int)((r + 1) * ntiles / nr);
+            int st = partials<CG, IG>(n, s);
+            if (st != FEWHA_OK) return st;
+            k_reduce_partials<<<(len + 31) / 32, 32 * RG, 0, s>>>(workspace, n, len, gw, gb, len - A.Cout, accumulate,
+                                                                  total, r > 0, r + 1 < nr);
+            if ((st = ck()) != FEWHA_OK) return st;
+        }
+        return FEWHA_OK;
+    }
     int run(float *gw, float *gb, int accumulate, float *workspace, cudaStream_t s)
     {
-        const int n = (int)(parts < WG_CTAS ? parts : WG_CTAS), Cin = A.Cin, Cout = A.Cout;  // n <= ntiles
-        A.part = workspace;
-        A.ntiles = (int)ntiles;
         // channel block: 32 x 32, or narrow on the side with at most 8 output / 4
         // input channels (the padding would be most of the work)
-        const int st = Cout <= 8  ? partials(k_conv3x3_wgrad_partial<2, 16>, wg_smem<2, 16>(), 8, 32, n, s)
-                       : Cin <= 4 ? partials(k_conv3x3_wgrad_partial<8, 2>, wg_smem<8, 2>(), 32, 4, n, s)
-                                  : partials(k_conv3x3_wgrad_partial<8, 16>, wg_smem<8, 16>(), 32, 32, n, s);
-        if (st != FEWHA_OK) return st;
-        const int len = Cout * Cin * 9 + Cout;
-        k_reduce_partials<<<(len + 31) / 32, 32 * RG, 0, s>>>(workspace, n, len, gw, gb, Cout * Cin * 9, accumulate);
-        return ck();
+        return A.Cout <= 8  ? gradient<2, 16>(gw, gb, accumulate, workspace, s)
+               : A.Cin <= 4 ? gradient<8, 2>(gw, gb, accumulate, workspace, s)
+                            : gradient<8, 16>(gw, gb, accumulate, workspace, s);
     }
 };
 

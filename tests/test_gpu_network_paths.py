@@ -1,4 +1,5 @@
 """Paths of the warm-start network beside the ones of test_gpu_learned.py."""
+import numpy as np
 import pytest
 
 torch = pytest.importorskip("torch")
@@ -63,3 +64,79 @@ def test_backward_after_replays_of_a_captured_forward():
         net.forward(x.data_ptr(), net.n, y, tensor_cores=True)
         net.backward(x.data_ptr(), net.n, gy)
         assert torch.equal(replayed[i], net.grad), i
+
+
+SPAN = 260 * 2.0 ** -24  # about as many FP32 additions one after another as a 16 x 16 tile has pixels, then FP64
+
+
+def constant_gradients(value, B, H, W):
+    """Weight gradient per tap and bias gradient of an input of ones and a constant output gradient."""
+    rows, cols = [H - 1, H, H - 1], [W - 1, W, W - 1]
+    return value * B * np.outer(rows, cols), value * B * H * W
+
+
+@pytest.mark.parametrize("B,Cin,Cout,side", [(512, 5, 9, 64), (512, 32, 5, 64), (512, 4, 32, 64), (152, 6, 12, 32),
+                                             (153, 6, 12, 32), (37, 40, 33, 72)])
+def test_weight_gradient_of_many_images(B, Cin, Cout, side):
+    """FP32 partial sums stay short however many images there are: an input of ones and a constant output
+    gradient, whose sums have a closed form and whose rounding errors add up instead of cancelling.  Many tiles per
+    partial, and on both sides of the line between one round of partials and several (1216 tiles of 16 x 8)."""
+    from paper_2011_06842_gb300 import build, load_library
+    build.build()
+    L = load_library()
+    hw = side * side
+    x = torch.ones(B, Cin, side, side, device="cuda")
+    g = torch.full((B, Cout, side, side), 0.1, device="cuda")
+    size = L.fewha_conv3x3_wgrad_workspace(Cin, Cout, B, side, side)
+    ws = torch.full((size + 64,), 7.0, device="cuda")
+    gw, gb = torch.zeros(Cout, Cin, 3, 3, device="cuda"), torch.zeros(Cout, device="cuda")
+    rw, rb = constant_gradients(float(g[0, 0, 0, 0]), B, side, side)
+    for times, accumulate in ((1, 0), (2, 1)):
+        assert L.fewha_conv3x3_bwd_weight(x.data_ptr(), Cin * hw, hw, Cin, g.data_ptr(), Cout * hw, hw, Cout, B, side,
+                                          side, gw.data_ptr(), gb.data_ptr(), accumulate, ws.data_ptr(),
+                                          torch.cuda.current_stream().cuda_stream) == 0
+        assert np.abs(gw.cpu().numpy() / (times * rw) - 1).max() < SPAN
+        assert np.abs(gb.cpu().numpy() / (times * rb) - 1).max() < SPAN
+    assert torch.all(ws[size:] == 7.0)  # nothing written past the workspace
+
+
+@pytest.mark.parametrize("offset", [0, 1])
+def test_network_gradient_of_many_images(offset):
+    """fewha_convnet_bwd with several rounds of partials in a workspace of the stated size, on either side of an
+    8-byte boundary: hidden layers of ones, a last convolution that passes channel 0 on, and a constant output
+    gradient have closed-form gradients of the second and third weights."""
+    import ctypes as C
+
+    from paper_2011_06842_gb300 import build, load_library
+    from paper_2011_06842_gb300.fewha import NET
+    build.build()
+    L = load_library()
+    groups = [(80, 64), (3, 32)]  # 2608 tiles
+    n = sum(c * s * s for c, s in groups)
+    dev = dict(device="cuda", dtype=torch.float32)
+    w = [torch.zeros(32, 4, 3, 3, **dev), torch.zeros(32, 32, 3, 3, **dev), torch.zeros(5, 32, 3, 3, **dev)]
+    w[2][0, :, 1, 1] = 1.0
+    b = [torch.zeros(k, **dev) for k in (32, 32, 5)]
+    gw, gb = [torch.zeros_like(t) for t in w], [torch.zeros_like(t) for t in b]
+    hidden = [[f(c, 32, s, s, **dev) for c, s in groups] for f in (torch.ones, torch.ones, torch.empty, torch.empty)]
+    N, off = NET(), 0
+    N.C0, N.C, N.C3, N.ngroups = 4, 32, 5, len(groups)
+    for i, (c, s) in enumerate(groups):
+        N.count[i], N.side[i], N.off[i] = c, s, off
+        off += c * s * s
+        for dst, buf in zip((N.h1, N.h2, N.g1, N.g2), hidden):
+            dst[i] = buf[i].data_ptr()
+    for i in range(3):
+        N.w[i], N.b[i], N.gw[i], N.gb[i] = (t[i].data_ptr() for t in (w, b, gw, gb))
+    x, gy = torch.ones(4, n, **dev), torch.full((5, n), 0.1, **dev)
+    size = min(152, sum(c * ((s + 15) // 16) ** 2 for c, s in groups)) * (32 * 32 * 9 + 32)
+    ws = torch.full((size + 64,), 7.0, **dev)
+    assert L.fewha_convnet_bwd(C.byref(N), x.data_ptr(), n, gy.data_ptr(), n, ws.data_ptr() + 4 * offset,
+                               torch.cuda.current_stream().cuda_stream) == 0
+    ref = [constant_gradients(float(gy[0, 0]), c, s, s) for c, s in groups]
+    rw, rb = sum(r[0] for r in ref), sum(r[1] for r in ref)
+    for got in (gw[1], gw[2]):
+        assert np.abs(got.cpu().numpy() / rw - 1).max() < SPAN
+    for got in (gb[1], gb[2]):
+        assert np.abs(got.cpu().numpy() / rb - 1).max() < SPAN
+    assert torch.all(ws[offset + size:] == 7.0) and torch.all(ws[:offset] == 7.0)
