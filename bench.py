@@ -436,7 +436,7 @@ def run_batched(args, flush):
     by_kind = {}
     for i, k in enumerate(kinds):
         by_kind.setdefault(k, {"ctas": best["ctas"][i], "round": best["rounds"][i] if best["rounds"] else 0,
-                               "wfs_tile": list(best["tiles"][i]), "pt_band_rows": list(best["bands"][i])})
+                               "wfs_tile": list(best["tiles"][i]), "pt_band_rows": list(best["bands"][i] or ()) or "automatic"})
     out = {"instances": len(inst), "mix": "24 x tiny (8 m, 16x16, 4 NGS, 2 x 32^2) + 24 x medium (16 m, 40x40, "
            "4 LGS, 5 x 64^2) + 16 x ELT (39 m, 84x84, 6 LGS, 9 layers)", "steps": K, "warmup": W,
            "timed": "CUDA-graph replay of the bound batched launch", "us_per_step": us_step,

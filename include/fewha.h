@@ -221,8 +221,12 @@ typedef struct {
 int fewha_get_launch_info(const void *handle, fewha_launch_info *out);
 
 /* Height of the P_g^T gather's work items (bands of layer rows): rows_large
- * on the layers of the largest grid, rows_small on the smaller ones (default
- * 8 and 4); each is capped so that a band has at most 1024 layer nodes.
+ * on the layers of the largest grid, rows_small on the smaller ones; each is
+ * capped so that a band has at most 1024 layer nodes.  They hold for every
+ * later launch of the handle.  A handle without such a call chooses itself:
+ * heights 8 and 4, and in a batch or fewha_apply_op_multi, where a group may
+ * have several bands per CTA, the tallest bands if those take it fewer rounds.
+ * fewha_auto_pt_bands returns to that choice.
  * Re-plans the band tables and the shared memory they need; FEWHA_ERR_GEOMETRY
  * (and the earlier plan kept) when the staged rows do not fit.  Waits for the
  * device to be idle (blocking); batches created before the call are refused
@@ -230,6 +234,7 @@ int fewha_get_launch_info(const void *handle, fewha_launch_info *out);
  * suffices.  A tuning knob (fewha autotuner); results do not depend on it
  * beyond rounding order.  The paper has no counterpart. */
 int fewha_set_pt_bands(void *handle, int rows_large, int rows_small);
+int fewha_auto_pt_bands(void *handle);
 
 /* Copies the diagonal of alpha*D (Sec. 3) or of J^{-1} (Sec. 4) to host memory (n doubles). */
 int fewha_get_prior(const void *handle, double *alpha_d_host);
@@ -317,9 +322,10 @@ int fewha_batch_create_rounds(void *const *handles, int n, const int *ctas, cons
  * fewha_batch_create for the instance's CTA count.  tiles may be NULL. */
 int fewha_batch_create_ex(void *const *handles, int n, const int *ctas, const int *rounds, const int *tiles,
                           void **batch_out);
-/* CTAs and WFS tiles (2 ints per instance) of a batch. */
+/* CTAs, WFS tiles (2 ints per instance) and P_g^T bands per instance of a batch. */
 int fewha_batch_ctas(const void *batch, int *ctas_out);
 int fewha_batch_tiles(const void *batch, int *tiles_out);
+int fewha_batch_pt_bands(const void *batch, int *bands_out);
 int fewha_batch_solve(void *batch, const void *const *slopes, void *const *c, const fewha_state *states,
                       const fewha_solve_opts *opts, fewha_stats *stats_dev, cudaStream_t stream);
 void fewha_batch_destroy(void *batch);

@@ -208,6 +208,14 @@ int fewha_set_pt_bands(void *handle, int rows_large, int rows_small)
     return h->w()->set_bands(rows_large, rows_small);
 }
 
+int fewha_auto_pt_bands(void *handle)
+{
+    if (!handle) return FEWHA_ERR_ARG;
+    Handle *h = static_cast<Handle *>(handle);
+    if (cudaSetDevice(h->device) != cudaSuccess) return FEWHA_ERR_CUDA;
+    return h->w()->auto_bands();
+}
+
 int fewha_get_prior(const void *handle, double *out)
 {
     if (!handle || !out) return FEWHA_ERR_ARG;
@@ -475,6 +483,14 @@ int fewha_batch_tiles(const void *batch, int *tiles_out)
         tiles_out[2 * i] = b->ty[i];
         tiles_out[2 * i + 1] = b->tx[i];
     }
+    return FEWHA_OK;
+}
+
+int fewha_batch_pt_bands(const void *batch, int *bands_out)
+{
+    if (!batch || !bands_out) return FEWHA_ERR_ARG;
+    const Batch *b = static_cast<const Batch *>(batch);
+    for (int i = 0; i < b->n; i++) bands_out[i] = b->impl[i]->group_bands(b->ncta[i], b->smem);
     return FEWHA_OK;
 }
 

@@ -627,8 +627,12 @@ struct ImplBase {
     // memory (no allocation); FEWHA_ERR_SCRATCH if `bytes` is too small.
     virtual int apply_in_scratch(const void *x, void *y, void *scratch, size_t bytes, cudaStream_t s) = 0;
     virtual void launch_info(fewha_launch_info *out) const = 0;
-    // P^T band heights (layer rows) on the largest and on the smaller layers
+    // P^T band heights (layer rows) on the largest and on the smaller layers, for every launch; and back to
+    // the library's choice
     virtual int set_bands(int rows_large, int rows_small) = 0;
+    virtual int auto_bands() = 0;
+    // P^T bands that a group of nct CTAs with sm bytes of shared memory runs
+    virtual int group_bands(int nct, size_t sm) const = 0;
 };
 
 template <typename T, typename S>
@@ -654,6 +658,7 @@ struct Impl : ImplBase {
     T *ll_nodal = nullptr;
     std::vector<void *> band_owned;  // device tables of the P^T bands (replaced by plan_bands)
     int band_rows_large = 0, band_rows_small = 0;
+    bool bands_set = false;  // by a caller (set_bands): they hold for every group
     // second P^T band plan, for groups with several bands per CTA: the tallest
     // bands (kBandOutputs outputs each).  A band takes a CTA about 7 us whatever its
     // size (staging and contraction latencies), so fewer rounds of bands are
@@ -717,8 +722,7 @@ struct Impl : ImplBase {
         return std::max(smem_for(ty, tx), few_usable() ? few_fixed : 0);
     }
 
-    // band heights that a caller set explicitly (set_bands) hold for every group
-    bool few_usable() const { return few_fixed > 0 && band_rows_large == kBandLarge && band_rows_small == kBandSmall; }
+    bool few_usable() const { return few_fixed > 0 && !bands_set; }
 
     // the P^T band plan for a group of nct CTAs with sm bytes of shared memory:
     // the one with fewer rounds
@@ -1140,7 +1144,23 @@ struct Impl : ImplBase {
             plan_bands(ol, os);  // keep the earlier plan
             return st;
         }
+        bands_set = true;
         return FEWHA_OK;
+    }
+
+    int auto_bands() override
+    {
+        CK(cudaDeviceSynchronize());  // the tables may be in use
+        const int st = plan_bands(kBandLarge, kBandSmall);
+        if (st == FEWHA_OK) bands_set = false;
+        return st;
+    }
+
+    int group_bands(int nct, size_t sm) const override
+    {
+        Geo<T> G = base.geo;
+        choose_bands(G, nct, sm);
+        return G.nbands;
     }
 
     void launch_info(fewha_launch_info *out) const override

@@ -109,6 +109,8 @@ def load_library(path=LIB_PATH):
     lib.fewha_store.restype = C.c_int
     lib.fewha_set_pt_bands.argtypes = [vp, C.c_int, C.c_int]
     lib.fewha_set_pt_bands.restype = C.c_int
+    lib.fewha_auto_pt_bands.argtypes = [vp]
+    lib.fewha_auto_pt_bands.restype = C.c_int
     lib.fewha_set_noise.argtypes = [vp, dp, C.c_int]
     lib.fewha_set_noise.restype = C.c_int
     lib.fewha_get_launch_info.argtypes = [vp, C.POINTER(LAUNCH_INFO)]
@@ -133,6 +135,8 @@ def load_library(path=LIB_PATH):
     lib.fewha_batch_ctas.restype = C.c_int
     lib.fewha_batch_tiles.argtypes = [vp, C.POINTER(C.c_int)]
     lib.fewha_batch_tiles.restype = C.c_int
+    lib.fewha_batch_pt_bands.argtypes = [vp, C.POINTER(C.c_int)]
+    lib.fewha_batch_pt_bands.restype = C.c_int
     lib.fewha_batch_create_ex.argtypes = [C.POINTER(vp), C.c_int, C.POINTER(C.c_int), C.POINTER(C.c_int),
                                           C.POINTER(C.c_int), C.POINTER(vp)]
     lib.fewha_batch_create_ex.restype = C.c_int
@@ -209,7 +213,7 @@ def exported_symbols():
             "fewha_deflate_warm_start", "fewha_mcao_create", "fewha_mcao_n_actuators", "fewha_mcao_fit",
             "fewha_mcao_destroy", "fewha_get_launch_info", "fewha_set_noise", "fewha_read_probe", "fewha_set_pt_bands",
             "fewha_batch_create_ex", "fewha_batch_tiles", "fewha_conv3x3_fwd_tc", "fewha_convnet_fwd_tc", "fewha_convnet_fwd",
-            "fewha_convnet_bwd", "fewha_store"]
+            "fewha_convnet_bwd", "fewha_store", "fewha_auto_pt_bands", "fewha_batch_pt_bands"]
 
 
 def make_geometry(geom, noise_w, precision="f64", tile=0, grid=0) -> GEOMETRY:
@@ -280,6 +284,7 @@ class Fewha:
         self.dtype = torch.float64 if precision == "f64" else torch.float32
         self.slope_dtype = {"f64": torch.float64, "f32": torch.float32, "bf16s": torch.bfloat16}[precision]
         self.n_layers = len(geom.layers)
+        self.pt_bands = None  # P^T band heights set by set_pt_bands(); None: the library's choice per launch
 
     def close(self):
         if getattr(self, "_h", None):
@@ -310,8 +315,14 @@ class Fewha:
                                               1 if refresh_precond else 0), "fewha_set_noise")
 
     def set_pt_bands(self, rows_large, rows_small):
-        """P^T gather band heights (layer rows) on the largest / smaller layers."""
+        """P^T gather band heights (layer rows) on the largest / smaller layers, for every later launch."""
         self._check(self.lib.fewha_set_pt_bands(self._h, int(rows_large), int(rows_small)), "fewha_set_pt_bands")
+        self.pt_bands = (int(rows_large), int(rows_small))
+
+    def auto_pt_bands(self):
+        """Back to the band heights the library chooses per launch, as before any set_pt_bands()."""
+        self._check(self.lib.fewha_auto_pt_bands(self._h), "fewha_auto_pt_bands")
+        self.pt_bands = None
 
     def launch_info(self):
         """Launch shape chosen at creation (fewha_get_launch_info) as a dict."""
@@ -591,6 +602,12 @@ class FewhaBatch:
         self.lib.fewha_batch_tiles(self._b, out)
         return [(out[2 * i], out[2 * i + 1]) for i in range(self.n)]
 
+    def pt_bands(self):
+        """P^T bands of every instance, as its group runs them."""
+        out = (C.c_int * self.n)()
+        self.lib.fewha_batch_pt_bands(self._b, out)
+        return list(out)
+
     def new_stats(self):
         return self._torch.zeros(self.n * STATS_BYTES, dtype=self._torch.uint8, device=self.device)
 
@@ -712,7 +729,8 @@ def autotune_batch(fewhas, step, candidates=None, reps=3, tiles=((8, 8), (16, 16
       2. WFS tile shape per class (`tiles`), in turn, keeping a change only
          when the step gets faster.
       3. P^T band heights per class (`bands`: rows on the largest and on the
-         smaller layers of the geometry), the same way (set on the handles).
+         smaller layers of the geometry), the same way (set on the handles),
+         against the heights the handles came with (None: the library's choice).
     The CTA cap is the device's SM count (one CTA of 512 threads per SM).
     Returns ({"ctas", "rounds", "tiles", "bands", "ms"}, timings): the best
     setting (the handles keep its band heights) and every timed candidate."""
@@ -780,9 +798,7 @@ def autotune_batch(fewhas, step, candidates=None, reps=3, tiles=((8, 8), (16, 16
     # stage 3: P^T band heights per class
     band = {}
     for k in classes:
-        f0 = fewhas[members[k][0]]
-        li = f0.launch_info()
-        cur = (li["pt_rows_large"], li["pt_rows_small"])
+        cur = fewhas[members[k][0]].pt_bands
         for bl in bands:
             if bl == cur:
                 continue
@@ -795,7 +811,10 @@ def autotune_batch(fewhas, step, candidates=None, reps=3, tiles=((8, 8), (16, 16
             if ms is not None and ms < best_ms:
                 best_ms, cur = ms, bl
         for i in members[k]:
-            fewhas[i].set_pt_bands(*cur)
+            if cur is None:
+                fewhas[i].auto_pt_bands()
+            else:
+                fewhas[i].set_pt_bands(*cur)
         band[k] = cur
     return ({"ctas": ctas, "rounds": rounds, "tiles": tl, "bands": [band[key[i]] for i in range(n)],
              "ms": best_ms}, timings)
