@@ -408,8 +408,8 @@ int fewha_conv3x3_fwd_tc(const float *in, long in_bs, long in_cs, int Cin, const
  * gy_cs); h1, h2 (hidden activations) and g1, g2 (their gradients) are arrays of
  * count[g] x C x side[g] x side[g].  fewha_convnet_fwd writes h1, h2 and y;
  * fewha_convnet_bwd reads them and writes g1, g2 and the parameter gradients gw,
- * gb of sum gy y; workspace: at least min(152, sum over groups of count
- * ceil(side / 16)^2) (C max(C, C0, C3) 9 + max(C, C3)) floats. */
+ * gb of sum gy y; workspace: fewha_convnet_workspace(net) floats (from C0, C, C3
+ * and the groups' counts and sides; 0 if they are not valid). */
 #define FEWHA_NET_GROUPS 8
 typedef struct fewha_net {
     int C0, C, C3, ngroups;
@@ -419,13 +419,14 @@ typedef struct fewha_net {
     const float *w[3], *b[3];
     float *gw[3], *gb[3];
 } fewha_net;
+long fewha_convnet_workspace(const fewha_net *net);
 int fewha_convnet_fwd(const fewha_net *net, const float *x, long x_cs, float *y, long y_cs, cudaStream_t s);
 int fewha_convnet_bwd(const fewha_net *net, const float *x, long x_cs, const float *gy, long gy_cs, float *workspace,
                       cudaStream_t s);
 /* fewha_convnet_fwd_tc: the network conv(C0 -> 32) ReLU conv(32 -> 32) ReLU
  *   conv(32 -> C3) in one launch, with the arithmetic of three
  *   fewha_conv3x3_fwd_tc calls; C0, C3 <= 16.  Image i of group g (count[g]
- *   images of side[g] x side[g], side <= 128; at most 8 groups; host arrays)
+ *   images of side[g] x side[g], side <= 128; at most FEWHA_NET_GROUPS; host arrays)
  *   starts off[g] + i side[g]^2 floats into a channel of in and out; in_cs and
  *   out_cs are the channel strides; out must not overlap in.  status_dev as in
  *   fewha_conv3x3_fwd_tc. */

@@ -309,7 +309,7 @@ constexpr int kNetC = 32;                  // hidden channels
 constexpr int kNetRows = 8;                // most output rows per CTA
 constexpr int kNetP = 130;                 // staged pixels per (row, channel group): x = -1 .. 128
 constexpr int kNetPlane = kNetP * 16;      // bytes of one (row, channel group)
-constexpr int kNetGroups = 8;              // most image sizes of one launch
+constexpr int kNetGroups = FEWHA_NET_GROUPS;  // most image sizes of one launch
 constexpr int kNetW1 = 9 * 2 * 4 * 128, kNetW2 = 9 * 4 * 4 * 128, kNetW3 = 9 * 4 * 2 * 128;  // weight images
 constexpr int kNetCols = 512;              // TMEM columns ((kNetRows + 4) x 32 used)
 constexpr int kNetBars = (kNetRows + 4) + (kNetRows + 2) + kNetRows;

@@ -53,7 +53,7 @@ constexpr int TP = TX + 4;  // pitch of a staged row: x0-1 .. x0+TX plus slack, 
 //
 // A launch covers up to kMaxGroups groups of equal-size images (the layers of
 // each size): a group of small images alone leaves most SMs idle.
-constexpr int kMaxGroups = 8;
+constexpr int kMaxGroups = FEWHA_NET_GROUPS;
 
 struct ConvGroup {
     const float *in, *mask;
@@ -732,6 +732,19 @@ static int net_args_ok(const fewha_net *N)
     for (int g = 0; g < N->ngroups; g++)
         if (N->count[g] < 1 || N->side[g] < 1 || N->off[g] < 0 || !N->h1[g] || !N->h2[g]) return 0;
     return 1;
+}
+
+long fewha_convnet_workspace(const fewha_net *N)
+{
+    if (!N || N->ngroups < 1 || N->ngroups > kMaxGroups || N->C0 < 1 || N->C < 1 || N->C3 < 1) return 0;
+    long tiles = 0;
+    for (int g = 0; g < N->ngroups; g++) {
+        if (N->count[g] < 1 || N->side[g] < 1) return 0;
+        const long t = (N->side[g] + TS - 1) / TS;
+        tiles += N->count[g] * t * t;
+    }
+    const int C = N->C > N->C3 ? N->C : N->C3, M = C > N->C0 ? C : N->C0;  // the largest gradient of the three
+    return (tiles < WG_CTAS ? tiles : WG_CTAS) * ((long)N->C * M * 9 + C);
 }
 
 int fewha_convnet_fwd(const fewha_net *N, const float *x, long x_cs, float *y, long y_cs, cudaStream_t s)

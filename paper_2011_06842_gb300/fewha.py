@@ -59,12 +59,15 @@ class OPTS(C.Structure):
                 ("rhs_in_state", C.c_int), ("pad", C.c_int), ("c_out", C.c_void_p)]
 
 
+NET_GROUPS = 8  # FEWHA_NET_GROUPS
+
+
 class NET(C.Structure):
     """fewha_net: the training network's groups and buffers."""
-    _fields_ = [("C0", C.c_int), ("C", C.c_int), ("C3", C.c_int), ("ngroups", C.c_int), ("count", C.c_int * 8),
-                ("side", C.c_int * 8), ("off", C.c_long * 8), ("h1", C.c_void_p * 8), ("h2", C.c_void_p * 8),
-                ("g1", C.c_void_p * 8), ("g2", C.c_void_p * 8), ("w", C.c_void_p * 3), ("b", C.c_void_p * 3),
-                ("gw", C.c_void_p * 3), ("gb", C.c_void_p * 3)]
+    _fields_ = ([("C0", C.c_int), ("C", C.c_int), ("C3", C.c_int), ("ngroups", C.c_int),
+                 ("count", C.c_int * NET_GROUPS), ("side", C.c_int * NET_GROUPS), ("off", C.c_long * NET_GROUPS)]
+                + [(k, C.c_void_p * NET_GROUPS) for k in ("h1", "h2", "g1", "g2")]
+                + [(k, C.c_void_p * 3) for k in ("w", "b", "gw", "gb")])
 
 
 class LAUNCH_INFO(C.Structure):
@@ -190,6 +193,8 @@ def load_library(path=LIB_PATH):
         getattr(lib, name).restype = C.c_int
     lib.fewha_conv3x3_wgrad_workspace.argtypes = [I, I, I, I, I]
     lib.fewha_conv3x3_wgrad_workspace.restype = C.c_long
+    lib.fewha_convnet_workspace.argtypes = [C.POINTER(NET)]
+    lib.fewha_convnet_workspace.restype = C.c_long
     lib.fewha_strerror.argtypes = [C.c_int]
     lib.fewha_strerror.restype = C.c_char_p
     for name in ("fewha_create", "fewha_get_prior", "fewha_get_precond", "fewha_apply_op",
@@ -213,7 +218,8 @@ def exported_symbols():
             "fewha_deflate_warm_start", "fewha_mcao_create", "fewha_mcao_n_actuators", "fewha_mcao_fit",
             "fewha_mcao_destroy", "fewha_get_launch_info", "fewha_set_noise", "fewha_read_probe", "fewha_set_pt_bands",
             "fewha_batch_create_ex", "fewha_batch_tiles", "fewha_conv3x3_fwd_tc", "fewha_convnet_fwd_tc", "fewha_convnet_fwd",
-            "fewha_convnet_bwd", "fewha_store", "fewha_auto_pt_bands", "fewha_batch_pt_bands"]
+            "fewha_convnet_bwd", "fewha_store", "fewha_auto_pt_bands", "fewha_batch_pt_bands",
+            "fewha_convnet_workspace"]
 
 
 def make_geometry(geom, noise_w, precision="f64", tile=0, grid=0) -> GEOMETRY:

@@ -27,10 +27,9 @@ import math
 
 import numpy as np
 
-from .fewha import NET, FewhaError, _stream_ptr, load_library
+from .fewha import NET, NET_GROUPS, FewhaError, _stream_ptr, load_library
 
 CHANNELS = (4, 32, 32, 5)
-TC_MAX_GROUPS = 8  # most layer sizes of one launch of the whole network
 N_DIR = 5
 
 
@@ -112,10 +111,9 @@ class ConvNet:
         self._tc_groups = ((C.c_int * ng)(*[cnt for _, cnt, _ in self.groups]),
                            (C.c_int * ng)(*[nl for _, _, nl in self.groups]),
                            (C.c_long * ng)(*[off for off, _, _ in self.groups]))
-        # every group's partial sums of a weight gradient in one launch
-        tiles = sum(cnt * ((nl + 15) // 16) ** 2 for _, cnt, nl in self.groups)
-        ws = max(ws, min(152, tiles) * (9 * c1 * max(c0, c2, c3) + max(c1, c2, c3)))
         self._net = None
+        if ng <= NET_GROUPS:  # every group's partial sums of a weight gradient in one launch
+            ws = max(ws, self.lib.fewha_convnet_workspace(C.byref(self._net_args())))
         self._hidden = True  # the last forward() left its hidden layers in h1, h2
         self.work = torch.empty(max(ws, 1), dtype=torch.float32, device=dev)
         self.loss_part = torch.zeros(512, dtype=torch.float64, device=dev)
@@ -138,8 +136,8 @@ class ConvNet:
         holds y): the network then runs layer by layer, because a block of that
         launch reads input rows beside those whose outputs another block writes."""
         c0, _, _, c3 = CHANNELS
-        if tensor_cores and len(self.groups) <= TC_MAX_GROUPS and not _overlap(x_ptr, x_cs, c0, y.data_ptr(),
-                                                                               y.stride(0), c3, self.n):
+        if tensor_cores and len(self.groups) <= NET_GROUPS and not _overlap(x_ptr, x_cs, c0, y.data_ptr(),
+                                                                            y.stride(0), c3, self.n):
             p = lambda k: self._p(self.param, k)  # noqa: E731
             self._ck(self.lib.fewha_convnet_fwd_tc(C.c_void_p(x_ptr), x_cs, c0, p("w1"), p("b1"), p("w2"), p("b2"),
                                                    p("w3"), p("b3"), C.c_void_p(y.data_ptr()), y.stride(0), c3,
@@ -148,7 +146,7 @@ class ConvNet:
             self._hidden = False
             return y
         self._hidden = True
-        if not tensor_cores and len(self.groups) <= TC_MAX_GROUPS:
+        if not tensor_cores and len(self.groups) <= NET_GROUPS:
             self._ck(self.lib.fewha_convnet_fwd(C.byref(self._net_args()), C.c_void_p(x_ptr), x_cs,
                                                 C.c_void_p(y.data_ptr()), y.stride(0), _stream_ptr(self.torch)),
                      "convnet")
@@ -218,7 +216,7 @@ class ConvNet:
             for i, (name, _, launch) in enumerate(self.convolutions(x_ptr, x_cs, gy, tensor_cores=True)):
                 if i % 3 < 2:  # the two hidden layers of each group
                     self._ck(launch(), name)
-        if len(self.groups) <= TC_MAX_GROUPS:
+        if len(self.groups) <= NET_GROUPS:
             self._ck(lib.fewha_convnet_bwd(C.byref(self._net_args()), C.c_void_p(x_ptr), x_cs,
                                            C.c_void_p(gy.data_ptr()), gy.stride(0), work, s), "convnet backward")
             return
