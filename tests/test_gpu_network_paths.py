@@ -140,3 +140,52 @@ def test_network_gradient_of_many_images(offset):
     for got in (gb[1], gb[2]):
         assert np.abs(got.cpu().numpy() / rb - 1).max() < SPAN
     assert torch.all(ws[offset + size:] == 7.0) and torch.all(ws[:offset] == 7.0)
+
+
+@pytest.mark.parametrize("runs", [8, 9, 16])
+def test_many_runs_of_layer_sizes(runs):
+    """As many runs of equal-size layers as one launch takes, and more (layer by layer then): forward and every
+    parameter gradient against the FP64 oracle (FP32 1e-5 and 1e-4, as for two runs), and the tensor-core forward
+    within bfloat16's reach of it (1e-2 of the norm, as for a single convolution).  The gradients after that
+    forward belong to its own hidden layers: the oracle's gradients from those, again 1e-4."""
+    from oracle import learned as OL
+    layers = [configs.Layer(500.0 * i, 1.0 / runs, (16, 8)[i % 2], 2) for i in range(runs)]
+    geom = configs.Geometry("runs", D=2.0, obstruction=0.0, n_sub=4, gs=[configs.GuideStar(0.0, 0.0)], layers=layers,
+                            r0=0.2, wind=[(10.0, 0.1)] * runs)
+    net = network(geom)
+    assert len(net.groups) == runs
+    rng = np.random.default_rng(12)
+    x, gy = rng.standard_normal((4, net.n)), rng.standard_normal((5, net.n))
+    xd, gd = (torch.tensor(a, dtype=torch.float32, device="cuda") for a in (x, gy))
+    p, ref = net.params_numpy(), np.zeros((5, net.n))
+
+    def gradients(hidden):
+        total = {}
+        for (off, cnt, nl), h in zip(net.groups, hidden):
+            span = slice(off, off + nl * nl)
+            parts = OL.net_backward(x[:, span].reshape(1, 4, nl, nl), p, h, gy[:, span].reshape(1, 5, nl, nl))
+            for k, g in parts.items():
+                total[k] = total.get(k, 0.0) + g
+        return total
+
+    hidden = []
+    for off, cnt, nl in net.groups:
+        out, h = OL.net_forward(x[:, off:off + nl * nl].reshape(1, 4, nl, nl), p)
+        ref[:, off:off + nl * nl] = out.reshape(5, -1)
+        hidden.append(h)
+    exact = gradients(hidden)
+
+    def rel(a, b):
+        return np.linalg.norm(a - b) / np.linalg.norm(b)
+
+    y = torch.full((5, net.n), 7.0, device="cuda")
+    for tensor_cores, tol in ((False, 1e-5), (True, 1e-2), (False, 1e-5)):
+        net.forward(xd.data_ptr(), net.n, y, tensor_cores=tensor_cores)
+        assert rel(y.double().cpu().numpy(), ref) < tol
+        net.backward(xd.data_ptr(), net.n, gd)
+        got = net.grad.double().cpu().numpy()
+        grads = exact
+        if tensor_cores:
+            grads = gradients([(a.double().cpu().numpy(), b.double().cpu().numpy()) for a, b in zip(net.h1, net.h2)])
+        for name, (o, shape) in net.offsets.items():
+            assert rel(got[o:o + int(np.prod(shape))].reshape(shape), grads[name]) < 1e-4, (name, tensor_cores)
