@@ -203,8 +203,9 @@ double fewha_layer_spacing(const void *handle, int layer);
  * geometry's `grid` fixed them), threads per CTA, dynamic shared memory, and
  * which forms of the operator phases run: split_levels = 1 when the finest
  * wavelet level is tiled over all CTAs and only the coarser levels stay on
- * one CTA per layer (at least twice as many CTAs as layers), 0 when each
- * layer's CTA runs every level; staged_tables = 1 when the P_g^T gather
+ * one CTA per layer (at least twice as many CTAs as layers, and a layer above
+ * 32 x 32 nodes for FEWHA_F64, above 64 x 64 otherwise), 0 when each layer's CTA
+ * runs every level; staged_tables = 1 when the P_g^T gather
  * stages its interpolation-weight tables in shared memory beside the adjoint
  * wavefront rows, 0 when it reads them from global memory; the WFS tile
  * shape; the P_g^T work items (bands of layer rows) and the adjoint wavefront
@@ -361,8 +362,10 @@ int fewha_batch_launch(void *batch, cudaStream_t stream);
  *   applied to gout.  fewha_conv3x3_bwd_data_relu: the same, then 0 where
  *   act <= 0 (act laid out like gin, the ReLU output; NULL: no mask).
  * fewha_conv3x3_bwd_weight: gw (Cout x Cin x 9) and gb (Cout) of
- *   sum_b,co,y,x gout * out; written, or added when accumulate != 0;
- *   workspace: fewha_conv3x3_wgrad_workspace(...) floats; deterministic.
+ *   sum_b,co,y,x gout * out; written, or added when accumulate != 0; FP32 sums
+ *   of about 256 products, the rest in FP64; workspace:
+ *   fewha_conv3x3_wgrad_workspace(...) floats; deterministic.  324 Cin + 256
+ *   Cout <= 51200 (FEWHA_ERR_ARG otherwise).
  * fewha_relu_bwd: g[i] = 0 where act[i] <= 0 (act = the ReLU output).
  * fewha_mse_grad: grad = 2 (pred - target) / n; loss_part512[512] partial sums
  *   of (pred - target)^2 (the loss is their sum / n).
@@ -524,8 +527,9 @@ void fewha_mcao_destroy(void *mcao);
  * device (no cached pointer outlives a device reset); the current device must
  * be the handle's (FEWHA_ERR_ARG otherwise).  Problems whose buffers do not
  * fit are rejected with FEWHA_ERR_SCRATCH (an ELT-size FP64 operator, n =
- * 98304 with 6 sensors of 84 x 84 subapertures, counts as about 4.8 MB, of
- * which 3 MB are reserved for partial sums).
+ * 98304 with 6 sensors of 84 x 84 subapertures, counts as about 4.8 MB: 3 MB
+ * of the test are partial sums, which the operator no longer stores, so that the
+ * same problems are refused as ever).
  * All calls share the one array, which keeps the last call's contents: calls
  * that overlap on the GPU (different streams, different handles on the same
  * device) race and must be ordered by the caller.  The paper has no

@@ -624,8 +624,6 @@ __device__ __forceinline__ Taps<T, L> load_taps(const Geo<T> &G)
     return tp;
 }
 
-// One run of `run` output pairs starting at pair m0 of the line at base
-// (element stride es), into out[0 .. 2 kRun).
 // One tap pair of a synthesis sum.  FP64: two FMAs instead of a product, an FMA
 // and an addition.
 template <typename T>
@@ -633,8 +631,9 @@ __device__ __forceinline__ void synth_acc(T &x, T h, T a, T g, T d)
 {
     x = fma(g, d, fma(h, a, x));
 }
-// RUN > 0: `run` is that constant, and only its pairs are computed.  FP64 sums
-// are FMA chains: two FP64 instructions per tap pair instead of three.
+// One run of `run` output pairs starting at pair m0 of the line at base
+// (element stride es), into out[0 .. 2 kRun).  RUN > 0: `run` is that constant,
+// and only its pairs are computed.
 template <typename T, int L, bool SYNTH, int RUN = 0>
 __device__ __forceinline__ void dwt_run(const T *base, int es, int N, int half, int run_, int m0,
                                         const Taps<T, L> &tp, T (&out)[2 * kRun])

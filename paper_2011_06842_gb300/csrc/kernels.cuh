@@ -956,11 +956,17 @@ struct Impl : ImplBase {
             const long h = P.geom.layers[l].n / 2;
             G.ll_off[l + 1] = G.ll_off[l] + h * h;
         }
-        // The split form costs an iteration two phases and two barriers, 4.4 us
-        // each in FP32 and 7 to 10 us in FP64 on 152 CTAs; the finest level on
-        // the layer's own CTA costs about 2 us at 64^2 in FP32 and 3 us at 32^2
-        // in FP64 (twice FP32's next size, and four times FP64's, is more than
-        // the phase).
+        // The split form costs an iteration two phases and two barriers (on 152 CTAs
+        // 4.4 us in FP32, 7 to 10 us in FP64) and takes the finest level and three
+        // quarters of the update off the layer CTAs.  By the largest layer, us a
+        // step of six iterations whole / split, recycling the last direction and
+        // all eight:
+        //   FP32   32^2  194 / 235, 268 / 313     64^2  237 / 269, 326 / 343
+        //         128^2  395 / 341, 559 / 432
+        //   FP64   32^2  321 / 344, 557 / 570     64^2  620 / 445, 930 / 681
+        //         128^2 1816 / 639, 2446 / 908
+        // With all of 16 directions the first three are 897 / 1041, 1141 / 1139 and
+        // (FP64 32^2) 1829 / 1816 us for 18 iterations.
         {
             int nmax = 0;
             for (int l = 0; l < P.L; l++) nmax = std::max(nmax, P.geom.layers[l].n);
@@ -1577,8 +1583,9 @@ struct Impl : ImplBase {
         const size_t o_ll = up256(o_u + (size_t)P.n * sizeof(T));
         const size_t o_wq = std::is_same<T, S>::value ? 0 : up256(o_ll + ll_elems() * sizeof(T));
         const size_t need = std::max(up256(o_ll + ll_elems() * sizeof(T)), up256(o_wq + (size_t)P.n * sizeof(T)));
-        // the size test of the entry point's contract: record, partial sums of
-        // every CTA, nodal layers, adjoint wavefronts and P^T output
+        // the size test of the entry point's contract (fewha.h): a record, partial
+        // sums of every CTA, nodal layers, adjoint wavefronts and P^T output; the
+        // first two are counted and no longer stored
         const size_t contract = up256(sizeof(Record)) + up256((size_t)kSlots * kMaxCtas * sizeof(double)) +
                                 up256(o_u + (size_t)P.n * sizeof(T));
         if (contract > bytes || need > bytes) return FEWHA_ERR_SCRATCH;

@@ -31,7 +31,7 @@ constexpr int PX = 4;     // adjacent pixels per thread
 constexpr int CO_T = 8;   // output channels per block
 constexpr int CI_T = 4;   // input channels staged per step
 constexpr int NT = TX * TY / PX;
-constexpr int CONV_CTAS = 6;  // CTAs per SM (registers and shared memory allow them)
+constexpr int CONV_CTAS = 6;  // CTAs per SM: 78 registers a thread (85 would fit) and 23 KB each
 constexpr int TP = TX + 4;  // pitch of a staged row: x0-1 .. x0+TX plus slack, 16-byte rows
 
 // out[b][co][y][x] = act(bias[co] + sum_ci sum_{ky,kx} w[co][ci][ky][kx] in[b][ci][y+ky-1][x+kx-1])
@@ -713,6 +713,7 @@ int fewha_conv3x3_bwd_weight(const float *in, long in_bs, long in_cs, int Cin, c
     if (!in || !gout || !gw || !gb || !workspace || Cin < 1 || Cout < 1 || B < 1 || H < 1 || W < 1)
         return FEWHA_ERR_ARG;
     const long tiles = (long)((W + TS - 1) / TS) * ((H + TS - 1) / TS) * B;
+    // the call's size limit (fewha.h): a whole tile's inputs and gradients in 200 KB
     const size_t smem = ((size_t)Cin * (TS + 2) * (TS + 2) + (size_t)Cout * TS * TS) * sizeof(float);
     if (smem > 200 * 1024 || tiles > 0x7fffffffL) return FEWHA_ERR_ARG;
     WgradLaunch L(Cin, Cout);

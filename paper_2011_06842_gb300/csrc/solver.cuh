@@ -254,8 +254,9 @@ __device__ __forceinline__ void phase_init(const Args<T, S> &A, const Basis &b, 
 // about two FP64 FMAs per clock (8 operations per element of the update, 12 per
 // element and level of the transform): with the 64^2 block of a 128^2 layer UA1
 // took 57 us and D2E 45, with the 32^2 block 26 and 22 (15 and 13.5 with the runs
-// of dwt_pass), for one more tiled phase and barrier on each side (3.7 + 1 us).  In FP32 the block is latency
-// bound and a phase with its barrier costs more than the level saves.
+// of dwt_pass), for one more tiled phase and barrier on each side (3.7 + 1 us).
+// In FP32 the block is latency bound and a phase with its barrier costs more than
+// the level saves.
 template <typename T>
 __device__ __forceinline__ int split_depth(const Geo<T> &G)
 {
@@ -287,15 +288,14 @@ __device__ __forceinline__ void for_detail_vectors(const Geo<T> &G, long lo, lon
 
 // Two ways to run the layers' transforms, chosen per instance:
 //   split (at least twice as many CTAs as layers, and layers large enough,
-//     Geo::split_min): the finest level is tiled
-//     over all CTAs (A2, D1); the first L CTAs own one layer's (n/2)^2 block
-//     each, run its coarser levels in shared memory and take no detail
-//     coefficients (the block transforms are then the critical path);
+//     Geo::split_min): the finest level, or two (split_depth), is tiled over all
+//     CTAs (A2, D1); the first L CTAs own one layer's approximation block each,
+//     run its coarser levels in shared memory and take no detail coefficients
+//     (the block transforms are then the critical path);
 //   whole (fewer CTAs, e.g. the small instances of a batch, or smaller layers):
-//     each layer's CTA
-//     updates the whole layer, runs every level in shared memory and updates
-//     the layer again after the forward transform; A2 and D1 are empty, so an
-//     iteration has four grid barriers instead of six.
+//     each layer's CTA updates the whole layer, runs every level in shared
+//     memory and updates the layer again after the forward transform; A2 and D1
+//     are empty, so an iteration has four grid barriers instead of six.
 template <typename T, typename S>
 __device__ __forceinline__ bool split_levels(const Args<T, S> &A)
 {
@@ -605,8 +605,8 @@ __device__ __forceinline__ bool phase_C(const Args<T, S> &A, const Basis &b, int
 // the smaller tile keeps as many CTAs busy).
 constexpr int kFineTile = 16, kFineTile2 = 8;
 
-// Work item w -> layer l and tile origin (in coefficient pairs); false past the end.
-// of level LV (0 = finest)
+// Work item w -> layer l and tile origin (in coefficient pairs) of level LV (0 =
+// finest); false past the end.
 template <int LV, typename T>
 __device__ __forceinline__ bool fine_tile(const Geo<T> &G, int w, int &l, int &p0y, int &p0x)
 {

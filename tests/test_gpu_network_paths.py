@@ -189,3 +189,17 @@ def test_many_runs_of_layer_sizes(runs):
             grads = gradients([(a.double().cpu().numpy(), b.double().cpu().numpy()) for a, b in zip(net.h1, net.h2)])
         for name, (o, shape) in net.offsets.items():
             assert rel(got[o:o + int(np.prod(shape))].reshape(shape), grads[name]) < 1e-4, (name, tensor_cores)
+
+
+@pytest.mark.parametrize("name", ["micro", "mixed", "elt"])
+def test_one_launch_has_the_bits_of_three(name):
+    """The whole network on the tensor cores in one launch adds the same products in the same order as its
+    convolutions one by one."""
+    net = network(configs.get(name))
+    g = torch.Generator(device="cuda").manual_seed(1)
+    x = torch.randn(4, net.n, generator=g, device="cuda")
+    y, z = torch.empty(5, net.n, device="cuda"), torch.empty(5, net.n, device="cuda")
+    net.forward(x.data_ptr(), net.n, y, tensor_cores=True)
+    for conv, _, launch in net.convolutions(x.data_ptr(), net.n, z, tensor_cores=True):
+        assert launch() == 0, conv
+    assert torch.equal(y, z)
