@@ -226,7 +226,7 @@ int fewha_get_launch_info(const void *handle, fewha_launch_info *out);
  * capped so that a band has at most 1024 layer nodes.  They hold for every
  * later launch of the handle.  A handle without such a call chooses itself:
  * heights 8 and 4, and in a batch or fewha_apply_op_multi, where a group may
- * have several bands per CTA, the tallest bands if those take it fewer rounds.
+ * have several bands per CTA, the tallest bands if they are expected to be faster.
  * fewha_auto_pt_bands returns to that choice.
  * Re-plans the band tables and the shared memory they need; FEWHA_ERR_GEOMETRY
  * (and the earlier plan kept) when the staged rows do not fit.  Waits for the

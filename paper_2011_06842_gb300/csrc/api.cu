@@ -443,7 +443,7 @@ int fewha_batch_create_ex(void *const *handles, int n, const int *ctas, const in
         } else if ((st = b->impl[i]->tiles_for(b->ncta[i], &b->ty[i], &b->tx[i]))) {
             return st;
         }
-        b->smem = std::max(b->smem, b->impl[i]->smem_want(b->ty[i], b->tx[i]));
+        b->smem = std::max(b->smem, b->impl[i]->smem_want(b->ty[i], b->tx[i], b->ncta[i], false));
     }
     b->total = *std::max_element(used.begin(), used.end());
     if ((st = b->impl[0]->batch_capacity(b->smem, &cap))) return st;

@@ -614,8 +614,9 @@ struct ImplBase {
     // WFS tile shape for a group of `ctas` CTAs, and the dynamic shared memory it needs
     virtual int tiles_for(int ctas, int *ty, int *tx) const = 0;
     virtual size_t smem_for(int ty, int tx) const = 0;
-    // the same, with what a faster plan for small groups needs (at creation of a batch)
-    virtual size_t smem_want(int ty, int tx) const = 0;
+    // the same, with what a faster plan needs if a group of nct CTAs runs it (a
+    // batch's solver, or the operator chain)
+    virtual size_t smem_want(int ty, int tx, int nct, bool chain) const = 0;
     // host copy of this instance's kernel arguments for one time step
     virtual int batch_args(void *out, const void *sl, void *c, const fewha_state *st, const fewha_solve_opts *o,
                            fewha_stats *stats, int cta0, int ncta, int ty, int tx, size_t smem) const = 0;
@@ -659,14 +660,22 @@ struct Impl : ImplBase {
     std::vector<void *> band_owned;  // device tables of the P^T bands (replaced by plan_bands)
     int band_rows_large = 0, band_rows_small = 0;
     bool bands_set = false;  // by a caller (set_bands): they hold for every group
-    // second P^T band plan, for groups with several bands per CTA: the tallest
-    // bands (kBandOutputs outputs each).  A band takes a CTA about 7 us whatever its
-    // size (staging and contraction latencies), so fewer rounds of bands are
-    // faster: 9 ELT layers on 9 CTAs take 16 rounds of 8- and 4-row bands.  A batch of
-    // 24 tiny, 24 medium and 16 ELT instances: 2425 us with one plan, 2270 with two.
+    // Second P^T band plan, for groups with several bands per CTA: the tallest
+    // bands (kBandOutputs outputs each).  Staging and contracting one pass of a band
+    // (the guide stars whose pupil rows fit at once) takes a CTA about 3.2 us in FP32
+    // and 3.8 us in FP64, and every adjoint value it stages 1.3 and 2.6 ns more, so a
+    // pass costs as much as kPassValues values (within 20 % on one CTA, band heights
+    // 2 to 128, 7 geometries; a 16-row band of a 64^2 ELT layer takes 14 us, its four
+    // 4-row bands 19).  A batch of 24 tiny, 24 medium and 16 ELT instances: 2425 us
+    // with one plan, 2270 with two.
+    static constexpr int kPassValues = sizeof(T) == 8 ? 1500 : 2500;
     Geo<T> few{};
     std::vector<void *> few_owned;
     size_t few_fixed = 0;  // its sm_fixed; 0: no such plan
+    std::vector<long> band_cost;  // of the bands of the last plan, in staged values
+    // by the CTAs of a group (from 0): whether it runs the second plan in the
+    // solver and in the operator chain (choose_plans)
+    std::vector<char> few_solver, few_chain;
 
     explicit Impl(const Plan &p) : P(p) {}
 
@@ -716,20 +725,48 @@ struct Impl : ImplBase {
     }
 
     size_t smem_for(int ty, int tx) const override { return std::max(sm_fixed, wfs_bytes(ty, tx)); }
-    // with room for the second band plan
-    size_t smem_want(int ty, int tx) const override
+    // with room for the second band plan if the group runs it (shared memory that
+    // is not needed costs L1 cache: 3 % of an ELT step on 72 CTAs)
+    size_t smem_want(int ty, int tx, int nct, bool chain) const override
     {
-        return std::max(smem_for(ty, tx), few_usable() ? few_fixed : 0);
+        return std::max(smem_for(ty, tx), few_wanted(nct, chain) ? few_fixed : 0);
     }
 
-    bool few_usable() const { return few_fixed > 0 && !bands_set; }
-
-    // the P^T band plan for a group of nct CTAs with sm bytes of shared memory:
-    // the one with fewer rounds
-    void choose_bands(Geo<T> &G, int nct, size_t sm) const
+    bool few_wanted(int nct, bool chain) const
     {
-        auto rounds = [&](int nb) { return (nb + nct - 1) / nct; };
-        if (!few_usable() || few_fixed > sm || rounds(few.nbands) >= rounds(G.nbands)) return;
+        const std::vector<char> &v = chain ? few_chain : few_solver;
+        return !bands_set && nct < (int)v.size() && v[nct];
+    }
+
+    // Which groups run the second plan: those whose CTAs then have fewer bands and
+    // whose busiest CTA does not take longer (to 2 %, the model's reach).  Fewer
+    // bands alone are not enough: LTAO on 36 CTAs 855 us a step with 8- and 4-row
+    // bands and 1012 with the tallest, ELT in FP64 on 48 CTAs 1175 and 1275, against
+    // 2248 and 1841 for the 16 m telescope on one CTA.  In the operator chain, where the
+    // gather is a kernel of its own, fewer bands win whenever the standard plan
+    // stages weight tables per band (ELT in FP64, 8 vectors: 352 and 319 us); without
+    // the tables the model holds there too (LTAO, 4 vectors: 112 and 129 us).
+    void choose_plans(const std::vector<long> &few_cost)
+    {
+        const Geo<T> &G = base.geo;
+        few_solver.assign(G.nbands + 1, 0);  // on more CTAs every band has its own
+        few_chain = few_solver;
+        for (int n = 1; n <= G.nbands; n++) {
+            if ((few.nbands + n - 1) / n >= (G.nbands + n - 1) / n) continue;
+            auto busiest = [n](const std::vector<long> &cost) {
+                std::vector<long> cta(n, 0);
+                for (size_t w = 0; w < cost.size(); w++) cta[w % n] += cost[w];
+                return *std::max_element(cta.begin(), cta.end());
+            };
+            few_solver[n] = busiest(few_cost) < 1.02 * busiest(band_cost);
+            few_chain[n] = G.stage_tab || few_solver[n];
+        }
+    }
+
+    // the P^T band plan for a group of nct CTAs with sm bytes of shared memory
+    void choose_bands(Geo<T> &G, int nct, size_t sm, bool chain) const
+    {
+        if (!few_wanted(nct, chain) || few_fixed > sm) return;
         G.nbands = few.nbands;
         G.band_layer = few.band_layer, G.band_row0 = few.band_row0, G.band_rows = few.band_rows;
         G.band_ilo = few.band_ilo, G.band_ihi = few.band_ihi;
@@ -807,6 +844,7 @@ struct Impl : ImplBase {
             }
         }
         G.nbands = (int)bl.size();
+        band_cost.assign(G.nbands, 0);
         std::vector<int> bilo((size_t)P.G * G.nbands), bihi((size_t)P.G * G.nbands);
         int max_rows = 1, max_rows_sum = 1;
         std::vector<int> rows_sum(G.nbands, 0);
@@ -825,6 +863,7 @@ struct Impl : ImplBase {
                 bilo[(size_t)g * G.nbands + w] = lo;
                 bihi[(size_t)g * G.nbands + w] = hi;
                 max_rows = std::max(max_rows, hi - lo);
+                band_cost[w] += (long)(hi - lo) * P.gm[g];
                 rows_sum[w] += hi - lo;
                 max_rows_sum = std::max(max_rows_sum, rows_sum[w]);
             }
@@ -853,6 +892,7 @@ struct Impl : ImplBase {
                         rows_tot += bihi[i] - bilo[i];
                     }
                     if (g1 == g0) return FEWHA_ERR_GEOMETRY;  // rows_chunk >= max_rows
+                    band_cost[w] += kPassValues;
                     for (int g = g0, c = 0, r = 0; g < g1; g++) {
                         const size_t i = (size_t)g * G.nbands + w;
                         gend[i] = g1;
@@ -1069,14 +1109,17 @@ struct Impl : ImplBase {
         smem = std::max(sm_layer, sm_wfs);
         sm_base = smem;
         sm_layer_ = sm_layer;
+        std::vector<long> few_cost;
         if ((st = plan_bands(FEWHA_MAX_GRID, FEWHA_MAX_GRID)) == FEWHA_OK) {
             few = G;
             few_owned.swap(band_owned);
             few_fixed = sm_fixed;
+            few_cost = band_cost;
         } else if (st != FEWHA_ERR_GEOMETRY) {
             return st;  // (too many rows for the shared memory: no second plan)
         }
         if ((st = plan_bands(kBandLarge, kBandSmall))) return st;
+        if (few_fixed > 0) choose_plans(few_cost);
         int dev, nsm;
         CK(cudaGetDevice(&dev));
         CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
@@ -1165,7 +1208,7 @@ struct Impl : ImplBase {
     int group_bands(int nct, size_t sm) const override
     {
         Geo<T> G = base.geo;
-        choose_bands(G, nct, sm);
+        choose_bands(G, nct, sm, false);
         return G.nbands;
     }
 
@@ -1546,7 +1589,7 @@ struct Impl : ImplBase {
         const int per = std::max(1, ncta / nvec);
         int ty, tx;
         if (tiles_for(per, &ty, &tx)) return FEWHA_ERR_GEOMETRY;
-        const size_t sm = smem_want(ty, tx);
+        const size_t sm = smem_want(ty, tx, per, true);
         MultiArgs<T, S> M{};
         M.per = per;
         for (int v = 0; v < nvec; v++) {
@@ -1562,7 +1605,7 @@ struct Impl : ImplBase {
             A.cta0 = v * per;
             A.ncta = per;
             set_tiles(A.geo, ty, tx);
-            choose_bands(A.geo, per, sm);
+            choose_bands(A.geo, per, sm, true);
             A.smem_bytes = sm;
             A.trace = nullptr;
             A.trace_cap = 0;
@@ -1650,7 +1693,7 @@ struct Impl : ImplBase {
         A.cta0 = cta0;
         A.ncta = nct;
         set_tiles(A.geo, ty, tx);
-        choose_bands(A.geo, nct, sm);
+        choose_bands(A.geo, nct, sm, false);
         A.smem_bytes = sm;
         A.trace = nullptr;
         A.trace_cap = 0;

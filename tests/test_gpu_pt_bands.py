@@ -101,3 +101,18 @@ def test_autotuner_keeps_the_automatic_heights_apart(lib):
     batch.close()
     for f in handles:
         f.close()
+
+
+@pytest.mark.parametrize("name,prec,ctas,taller", [("ltao", "f32", 36, False), ("elt", "f64", 48, False),
+                                                   ("elt", "f32", 40, False), ("elt", "f32", 9, True),
+                                                   ("elt", "f32", 152, False), ("medium", "f32", 2, True),
+                                                   ("medium", "f64", 20, True), ("tiny", "f64", 1, True)])
+def test_taller_bands_where_they_pay(lib, name, prec, ctas, taller):
+    """The library's choice on both sides of the line (each side was timed with both plans)."""
+    geom = configs.get(name)
+    f = lib.Fewha(geom, np.ones(len(geom.gs)), prec)
+    batch = lib.FewhaBatch([f], [ctas])
+    standard = f.launch_info()["pt_bands"]
+    assert batch.pt_bands()[0] < standard if taller else batch.pt_bands()[0] == standard
+    batch.close()
+    f.close()
