@@ -37,7 +37,7 @@
  *  - Asynchrony: compute calls enqueue work on the given stream and return.
  *    Calls on one handle share its scratch memory, so those that overlap on
  *    the GPU (different streams) must be ordered by the caller.  Exception:
- *    fewha_rhs may overlap fewha_fit and fewha_mcao_fit (the next frame's
+ *    fewha_rhs may overlap one fewha_fit or fewha_mcao_fit (the next frame's
  *    right-hand side beside this frame's fitting).
  */
 #ifndef FEWHA_H
