@@ -1076,8 +1076,7 @@ struct Impl : ImplBase {
         if ((st = alloc((size_t)P.n, &base.nodal)) || (st = alloc((size_t)P.n, &base.u)) ||
             (st = alloc((size_t)P.n, &base.wq)) ||
             (st = alloc((size_t)P.psi_off[P.G], &base.psi)) || (st = alloc(ll_elems(), &base.ll)) ||
-            (st = alloc(ll_elems(), &ll_nodal)) || (st = alloc((size_t)kSlots * kMaxCtas, &base.part)) ||
-            (st = alloc((size_t)1, &base.rec)))
+            (st = alloc((size_t)kSlots * kMaxCtas, &base.part)) || (st = alloc((size_t)1, &base.rec)))
             return st;
         if constexpr (std::is_same<T, S>::value) {
             base.nodal_t = base.nodal;
@@ -1120,6 +1119,7 @@ struct Impl : ImplBase {
         }
         if ((st = plan_bands(kBandLarge, kBandSmall))) return st;
         if (few_fixed > 0) choose_plans(few_cost);
+        if ((st = alloc(ll_elems(), &ll_nodal))) return st;
         int dev, nsm;
         CK(cudaGetDevice(&dev));
         CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
